@@ -284,9 +284,9 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
     // narrow layers with long horizons: one warp per neuron, time scanned in parallel
     pl->tp = c.T >= kTpMinT && BN <= kTpMaxNeurons && tp_smem_bytes(c.T, c.K, true) <= kTpMaxSmem;
     // blocks of the forward and backward kernels that fit on one SM. The backward's is taken
-    // for the compartments-innermost layout and the build without dL/dbeta, so that both
-    // layouts and both builds of a layer share one tiling (and sum the parameter gradients
-    // in the same order).
+    // for the build without dL/dbeta, so that both builds of a layer share one tiling (and sum
+    // the parameter gradients in the same order); the two layouts of a layer share it only
+    // while a thread has one row (the paper layout's twin kernels fit other block counts).
     int res_f = 0, res_b = 0;
     if (!pl->tp && O > 0 && c.T > 0) {
         FwdArgs fa;
@@ -303,7 +303,7 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
             res_f = 0;
             (void)cudaGetLastError();
         }
-        if (dispatch_backward(c, 0, g.L, ba, 0, nullptr, &res_b) != cudaSuccess) {
+        if (dispatch_backward(c, pl->layout, g.L, ba, 0, nullptr, &res_b) != cudaSuccess) {
             res_b = 0;
             (void)cudaGetLastError();
         }

@@ -11,8 +11,9 @@
 // chunk and row boundaries: through a per-thread ring of shared-memory slots filled
 // by cp.async (the forward; the backward of multi-chunk rows), or a ring of
 // registers (the backward of rows of at most 4 steps). In the paper's (C_o, P, H, W)
-// layout a lane's compartments are H*W apart; when H*W is a multiple of 32 the
-// forward stages each warp's inputs together (dendsn_forward_staged_kernel).
+// layout a lane's compartments are H*W apart; when H*W is even most layers take the twin
+// kernels (dendsn_twin.cuh: two neighbouring neurons per thread), and the forward of 8
+// float32 compartments stages each warp's inputs together (dendsn_forward_staged_kernel).
 //
 // Forward (Eqs. methods-compartment .. methods-lif-fire): V^d, V^s and S stay in
 // registers across all T steps; the HBM traffic per step is the K inputs read and
@@ -1200,8 +1201,8 @@ dendsn_forward_kernel(const FwdArgs A) {
     }
 }
 
-// Forward in the paper's (C_o, P, H, W) layout with the inputs staged per warp. Used when a
-// lane serves a whole neuron (K <= 8) and H*W and the column tile are multiples of 32: a
+// Forward in the paper's (C_o, P, H, W) layout with the inputs staged per warp. Used for 8
+// float32 compartments when H*W and the column tile are multiples of 32: a
 // warp's 32 neurons are then 32 consecutive positions of one channel group, so compartment k
 // of all of them is one contiguous run of 32 elements. Each lane copies its share of the
 // warp's K runs with 16-byte cp.async into the slot [k][32 lanes] (one copy per lane per
@@ -1336,27 +1337,12 @@ template <int NT> constexpr int red_stride() { return NT + 1; }
 // Bytes of shared memory block_partials needs for NA1 gradient slots.
 constexpr size_t red_bytes(int NA1, int NT) { return sizeof(float) * (size_t)NA1 * (NT + 1); }
 
-// Per-channel partial sums of a block's parameter-gradient vectors v (one per thread,
-// [alpha KT | xi KT | zeta KTb | kappa KTb | beta]) in a fixed order: segmented warp
-// shuffles over the columns of one channel, then the run leaders in shared memory (red,
-// red_bytes(NA1, NT)), one partial per (block, channel) to `partials`.
-template <int KT, int G, int LPN, int NT, int NA1>
-__device__ __forceinline__ void block_partials(const Geometry &g, const ThreadPos &pos,
-                                               float (&v)[NA1], float *red, float *partials) {
+// The last stage of block_partials: each (channel, slot) of the block summed over the rows and
+// run leaders of the tile from red[slot * RS + (row * TXn + column) * LPN + lane], by NT threads.
+template <int KT, int G, int LPN, int NT, int RS, int NA1>
+__device__ __forceinline__ void block_sums(const Geometry &g, const float *red, float *partials) {
     constexpr int KTb = KT / G;
     constexpr int NA = NA1 - 1;
-    constexpr int RS = red_stride<NT>();
-    // stage 1: within a warp, columns of one channel come in aligned runs of g.seg
-    for (int d = 1; d < g.seg; d <<= 1) {
-#pragma unroll
-        for (int a = 0; a < NA1; ++a)
-            v[a] = __fadd_rn(v[a], __shfl_xor_sync(0xffffffffu, v[a], d * LPN));
-    }
-    // stage 2: run leaders meet in shared memory; red[a][tid] (reuses the history space)
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < NA1; ++a) red[a * RS + threadIdx.x] = v[a];
-    __syncthreads();
     const int ct = blockIdx.x % g.nCT;
     const int p0 = ct * g.TXn;
     const int p1 = min(p0 + g.TXn, g.P);            // exclusive
@@ -1385,6 +1371,28 @@ __device__ __forceinline__ void block_partials(const Geometry &g, const ThreadPo
         else slot = NP - 1;                                                     // beta
         out[lc * NP + slot] = sum;
     }
+}
+
+// Per-channel partial sums of a block's parameter-gradient vectors v (one per thread,
+// [alpha KT | xi KT | zeta KTb | kappa KTb | beta]) in a fixed order: segmented warp
+// shuffles over the columns of one channel, then the run leaders in shared memory (red,
+// red_bytes(NA1, NT)), one partial per (block, channel) to `partials`.
+template <int KT, int G, int LPN, int NT, int NA1>
+__device__ __forceinline__ void block_partials(const Geometry &g, const ThreadPos &pos,
+                                               float (&v)[NA1], float *red, float *partials) {
+    constexpr int RS = red_stride<NT>();
+    // stage 1: within a warp, columns of one channel come in aligned runs of g.seg
+    for (int d = 1; d < g.seg; d <<= 1) {
+#pragma unroll
+        for (int a = 0; a < NA1; ++a)
+            v[a] = __fadd_rn(v[a], __shfl_xor_sync(0xffffffffu, v[a], d * LPN));
+    }
+    // stage 2: run leaders meet in shared memory; red[a][tid] (reuses the history space)
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < NA1; ++a) red[a * RS + threadIdx.x] = v[a];
+    __syncthreads();
+    block_sums<KT, G, LPN, NT, RS, NA1>(g, red, partials);
 }
 
 template <int KT, int G>
@@ -2435,6 +2443,12 @@ dendsn_backward_rowpair_kernel(const BwdArgs A) {
     block_partials<KT, 1, LPN, NT>(g, pos, v, reinterpret_cast<float *>(sregion), A.partials);
 }
 
+}  // namespace dendsn
+
+#include "dendsn_twin.cuh"
+
+namespace dendsn {
+
 // ---------------------------------------------------------------- launchers
 // Dynamic shared memory above 48 KB needs an explicit opt-in per kernel.
 template <typename Kern>
@@ -2473,6 +2487,33 @@ cudaError_t launch_or_query(Kern kernel, const Args &a, int blocks, int threads,
 #endif
 }
 
+// Whether a call takes the twin kernels (paper layout, K > 1): pairs of neurons stay within a
+// channel run (even H*W) and their [T, B, N] elements (pointers a and b, element sizes sa and
+// sb) are aligned for one access per pair; x and grad_x always are (16-byte bases, even offsets).
+inline bool takes_twin(const Geometry &g, const void *a, const void *b, size_t sa, size_t sb) {
+    return g.inner % 2 == 0 && g.inner < (1 << 29) && (reinterpret_cast<uintptr_t>(a) % (2 * sa)) == 0 &&
+           (b == nullptr || (reinterpret_cast<uintptr_t>(b) % (2 * sb)) == 0);
+}
+// The layers whose backward stays on one neuron per thread (us here -> twin, GB300, H*W = 256
+// and 64 channels or as said). The identity with several compartments per branch: its square
+// roots and divisions are not paired (T = 29, G = 2, B = 64, H*W = 64: 330 -> 544). Four
+// compartments per branch in 8-step chunks: the four rescanned V^d spill (T = 5, B = 32:
+// 29 -> 33).
+template <int G, int PSI, int L>
+constexpr bool twin_backward() { return !(PSI == PSI_IDENTITY && G > 1) && !(G == 4 && L == 8); }
+// Float32 lanes of up to 4 compartments over several chunks: the chunk's buffers, checkpoints and
+// two-level sums leave room for two blocks per SM only (T = 29, K = 4, G = 2, B = 32: 134 ->
+// 139; T = 64 about equal). Lanes of 8 compartments need enough neurons to hide a unit loop
+// that a small layer sees as latency (K = 8, G = 2, float32: T = 127, 8192 neurons 68 -> 78,
+// 32768 neurons 133 -> 116; T = 64, 16384 neurons 34 -> 38, 32768 neurons 53 -> 45), and more
+// of them when much of a row is an incomplete chunk (bfloat16 T = 10: 131072 neurons 35 -> 39,
+// 524288 neurons 144 -> 140; T = 5: 131072 neurons 20 -> 20, 524288 neurons 72 -> 53).
+inline bool twin_pays(const Geometry &g, int KT, bool f32) {
+    if (KT < 8) return !(f32 && g.n_ck > 0);
+    const bool whole = g.T <= 4 ? g.T == 4 : (g.T == 6 || g.T % 8 == 0 || g.T >= 32);
+    return g.BN * (g.K / KT) > (whole ? 24576 : 131072);
+}
+
 template <int K, int G, int PSI, int XT, int LAYOUT>
 cudaError_t launch_forward(const FwdArgs &a, int blocks, cudaStream_t s, int *resident) {
     using T = typename XType<XT>::type;
@@ -2480,13 +2521,39 @@ cudaError_t launch_forward(const FwdArgs &a, int blocks, cudaStream_t s, int *re
     using XI = XIO<T, KT, LAYOUT>;
     constexpr size_t raw = sizeof(typename XI::Raw);
     constexpr int NT = fwd_threads(K);
-    if constexpr (LAYOUT == 1 && K >= 2 && K <= 8 && DENDSN_FWD_ASYNC) {
-        // the paper layout with warps of 32 consecutive positions: staged per warp
+    if constexpr (LAYOUT == 1 && K == 8 && XT == 0) {
+        // 8 float32 compartments, warps of 32 consecutive positions: staged per warp in 16-byte
+        // copies; the twin forward's 8-byte ones measured slower (T = 64, G = 2, 524288 neurons:
+        // 193 -> 210 us; T = 6, G = 1, 1048576 neurons: 37.5 -> 39.8 us)
         if (a.g.inner % 32 == 0 && a.g.TXn % 32 == 0) {
             const size_t smem = (size_t)kFwdDepth * NT * K * sizeof(T) +
                                 kappa_smem_bytes(a.p.mask_mode, K / G, NT);
             return launch_or_query(dendsn_forward_staged_kernel<K, G, PSI, T>, a, blocks, NT, smem,
                                    s, resident);
+        }
+    }
+    if constexpr (LAYOUT == 1 && K >= 2) {
+        using W = typename TwinIO<T>::W;
+        if (takes_twin(a.g, a.spikes, a.v_out, sizeof(T), sizeof(float))) {
+            if constexpr (XT == 1) {
+                auto chunked = [&](auto lc, auto full) {
+                    constexpr int LC = decltype(lc)::value;
+                    return launch_or_query(dendsn_forward_twin_chunk_kernel<K, G, PSI, LC, decltype(full)::value>, a,
+                                           blocks, kTwinFwdThreads,
+                                           sizeof(W) * KT * LC * twin_fwd_buffers<KT, LC>() * kTwinFwdThreads, s,
+                                           resident);
+                };
+                using l4 = std::integral_constant<int, 4>;
+                using l8 = std::integral_constant<int, 8>;
+                using yes = std::true_type;
+                using no = std::false_type;
+                if (a.g.T <= 4) return a.g.T == 4 ? chunked(l4{}, yes{}) : chunked(l4{}, no{});
+                if (a.g.T == 6) return chunked(std::integral_constant<int, 6>{}, yes{});
+                return a.g.T % 8 == 0 ? chunked(l8{}, yes{}) : chunked(l8{}, no{});
+            } else {
+                return launch_or_query(dendsn_forward_twin_kernel<K, G, PSI, T>, a, blocks, kTwinFwdThreads,
+                                       sizeof(W) * KT * kTwinFwdDepth * kTwinFwdThreads, s, resident);
+            }
         }
     }
     const size_t smem = ((DENDSN_FWD_ASYNC && XI::kAsync) ? raw * fwd_depth<T, typename XI::Raw>() * NT : 0) +
@@ -2526,6 +2593,33 @@ cudaError_t launch_backward(const BwdArgs &a, int blocks, cudaStream_t s, int *r
             const size_t rsm = red > rp ? red : rp;
             return a.want_beta ? go_smem(dendsn_backward_rowpair_kernel<PSI, LAYOUT, true>, rsm)
                                : go_smem(dendsn_backward_rowpair_kernel<PSI, LAYOUT, false>, rsm);
+        }
+    }
+    // the paper layout with an even H*W: two neighbouring neurons per thread
+    if constexpr (LAYOUT == 1 && K >= 2 && twin_backward<G, PSI, L>()) {
+        if (takes_twin(a.g, a.gs, nullptr, sizeof(T), 0) && twin_pays(a.g, KT, XT == 0)) {
+            constexpr int NTW = NT / 2;
+            auto twin = [&](auto lc, auto full) {
+                constexpr int LC = decltype(lc)::value;
+                const size_t use = TwinSmem<T, KT, G, LC>::bytes(a.g.n_ck > 0, row_totals<K, G, T, L>()) * NTW;
+                return launch_or_query(dendsn_backward_twin_kernel<K, G, PSI, T, L, LC, decltype(full)::value>, a,
+                                       blocks, NTW, red > use ? red : use, s, resident);
+            };
+            using yes = std::true_type;
+            using no = std::false_type;
+            if constexpr (L == 4 && KT < 8) {
+                const size_t use = TwinShort<T, KT>::kBytes * NTW;
+                auto kernel = a.g.T == 4 ? dendsn_backward_twin_short_kernel<K, G, PSI, T, true>
+                                         : dendsn_backward_twin_short_kernel<K, G, PSI, T, false>;
+                return launch_or_query(kernel, a, blocks, NTW, red > use ? red : use, s, resident);
+            } else if constexpr (L == 4) {
+                using l4 = std::integral_constant<int, 4>;
+                return a.g.T == 4 ? twin(l4{}, yes{}) : twin(l4{}, no{});
+            } else {
+                using l8 = std::integral_constant<int, 8>;
+                if (a.g.T == 6) return twin(std::integral_constant<int, 6>{}, yes{});
+                return a.g.T % 8 == 0 ? twin(l8{}, yes{}) : twin(l8{}, no{});
+            }
         }
     }
     // rows of one full chunk, a whole 8-compartment neuron per lane: the phased kernel
