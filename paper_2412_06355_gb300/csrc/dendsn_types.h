@@ -122,7 +122,7 @@ template <int K, int G, int PSI, int XT, int L, int LAYOUT>
 cudaError_t launch_backward(const BwdArgs &a, int blocks, cudaStream_t s, int *resident);
 cudaError_t launch_finalize(const FinArgs &a, cudaStream_t s);
 
-// Time-parallel kernels (tp_kernels.cu): one warp per neuron, for layers with at least
+// Time-parallel kernels (tp_kernels.cu): one block per neuron, for layers with at least
 // kTpMinT steps and at most kTpMaxNeurons neurons whose backward history fits in shared
 // memory. XT: 0 = float, 1 = bfloat16; psi and layout are runtime arguments.
 constexpr int kTpMinT = 256;
