@@ -94,6 +94,8 @@ def library_path() -> str:
 def load() -> ctypes.CDLL:
     """Load libdendsn.so, building it first when it is missing or stale."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build()
@@ -135,13 +137,14 @@ def _ptr(t: Optional[torch.Tensor]):
         raise ValueError("DendSN tensors must live on a CUDA device")
     if not t.is_contiguous():
         raise ValueError("DendSN tensors must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        # the current stream's handle, without building a torch.cuda.Stream on every call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def launch_count() -> int:
@@ -157,30 +160,37 @@ def dendsn_workspace_size(cfg: dendsn_config):
     return int(s.value), int(w.value)
 
 
-def _need(cfg, **tensors):
-    """Refuses on the host any tensor smaller than what the config makes the kernels touch."""
-    T, B, N, K, C, Kb = cfg.T, cfg.B, cfg.N, cfg.K, cfg.C, cfg.K // cfg.G
-    sx = 2 if cfg.x_dtype == BF16 else 4
-    elems = {"x": T * B * N * K * sx, "grad_x": T * B * N * K * sx,
-             "spikes": T * B * N * sx, "grad_spikes": T * B * N * sx,
-             "v_out": T * B * N * 4, "grad_v": T * B * N * 4,
+# Bytes a config makes the kernels touch in each tensor, by the config's value and the current
+# device (scratch_bytes follows the device's residency). Bounded: forgotten when it has grown.
+_needs = {}
+
+
+def _config_needs(cfg) -> dict:
+    key = (bytes(cfg), torch.cuda.current_device() if torch.cuda.is_initialized() else -1)
+    n = _needs.get(key)
+    if n is None:
+        T, B, N, K, C, Kb = cfg.T, cfg.B, cfg.N, cfg.K, cfg.C, cfg.K // cfg.G
+        sx = 2 if cfg.x_dtype == BF16 else 4
+        step = T * B * N
+        n = {"x": step * K * sx, "grad_x": step * K * sx, "spikes": step * sx,
+             "grad_spikes": step * sx, "v_out": step * 4, "grad_v": step * 4,
              "alpha": C * K * 4, "xi": C * K * 4, "grad_alpha": C * K * 4, "grad_xi": C * K * 4,
              "zeta": C * Kb * 4, "kappa": C * Kb * 4, "grad_zeta": C * Kb * 4,
              "grad_kappa": C * Kb * 4, "mask": (N if cfg.mask_per_neuron else C) * Kb,
              "grad_beta": C * 4}
-    sizes = None
+        n["saved"], n["scratch"] = dendsn_workspace_size(cfg)
+        if len(_needs) >= 256:
+            _needs.clear()
+        _needs[key] = n
+    return n
+
+
+def _need(cfg, **tensors):
+    """Refuses on the host any tensor smaller than what the config makes the kernels touch."""
+    needs = _config_needs(cfg)
     for name, t in tensors.items():
-        if t is None:
-            continue
-        if name in ("saved", "scratch"):
-            if sizes is None:
-                sizes = dict(zip(("saved", "scratch"), dendsn_workspace_size(cfg)))
-            need = sizes[name]
-        else:
-            need = elems[name]
-        have = t.numel() * t.element_size()
-        if have < need:
-            raise ValueError(f"{name}: {have} bytes, the config needs {need}")
+        if t is not None and t.nbytes < needs[name]:
+            raise ValueError(f"{name}: {t.nbytes} bytes, the config needs {needs[name]}")
 
 
 def dendsn_forward(cfg, x, alpha, xi, zeta, kappa, mask, spikes, v_out=None, saved=None,

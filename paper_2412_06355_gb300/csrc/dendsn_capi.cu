@@ -74,6 +74,42 @@ cudaError_t launch_finalize(const FinArgs &a, cudaStream_t s) {
 }
 
 namespace {
+struct SmemKey {
+    const void *kernel;
+    int device;
+};
+std::mutex g_smem_mutex;
+SmemKey g_smem_done[1024];
+int g_smem_n = 0;
+}  // namespace
+
+// Opts `kernel` in to all the dynamic shared memory a block can have, once per device.
+cudaError_t allow_all_smem(const void *kernel) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    // what this thread saw last, so that the usual call takes no lock
+    static thread_local SmemKey seen[64];
+    SmemKey &s = seen[(reinterpret_cast<uintptr_t>(kernel) >> 4) % 64];
+    if (s.kernel == kernel && s.device == dev) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(g_smem_mutex);
+    bool done = false;
+    for (int i = 0; i < g_smem_n && !done; ++i)
+        done = g_smem_done[i].kernel == kernel && g_smem_done[i].device == dev;
+    if (!done) {
+        int most = 0;
+        cudaFuncAttributes at;
+        if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+        if ((e = cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
+        if (e != cudaSuccess) return e;
+        if (g_smem_n < (int)(sizeof g_smem_done / sizeof g_smem_done[0])) g_smem_done[g_smem_n++] = SmemKey{kernel, dev};
+    }
+    s = SmemKey{kernel, dev};
+    return cudaSuccess;
+}
+
+namespace {
 struct ResidentKey {
     const void *kernel;
     int threads;
@@ -133,7 +169,7 @@ struct Plan {
     bool keep_vs;      // saved holds V^s [T][BN] for the single-chunk (phased) backward
     int sx;            // bytes per x element
     int layout;        // 0 compartments innermost, 1 the paper's layer layout
-    bool tp;           // the time-parallel kernels (one warp per neuron)
+    bool tp;           // the time-parallel kernels (one block per neuron)
 };
 
 int sm_count() {
@@ -228,9 +264,7 @@ cudaError_t dispatch_forward(const dendsn_config &cfg, int layout, const FwdArgs
 cudaError_t dispatch_backward(const dendsn_config &cfg, int layout, int L, const BwdArgs &a,
                               int blocks, cudaStream_t s, int *resident = nullptr);
 
-dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
-    if (cfg == nullptr) return fail(DENDSN_ERR_INVALID_ARG, "cfg is NULL");
-    const dendsn_config &c = *cfg;
+dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
     if (c.T < 0 || c.B < 0 || c.N < 0)
         return fail(DENDSN_ERR_INVALID_ARG, "negative size (T=%d B=%d N=%d)", c.T, c.B, c.N);
     if (c.C < 1 || c.inner < 1) return fail(DENDSN_ERR_INVALID_ARG, "C and inner must be >= 1");
@@ -281,7 +315,7 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
     tile_columns(pl->gb, bwd_threads(KTB), c.K / KTB);
     pl->sx = (c.x_dtype == DENDSN_BF16) ? 2 : 4;
     pl->layout = (c.K > 1 && c.inner > 1) ? c.layout : 0;   // otherwise the layouts coincide
-    // narrow layers with long horizons: one warp per neuron, time scanned in parallel
+    // narrow layers with long horizons: one block per neuron, time scanned in parallel
     pl->tp = c.T >= kTpMinT && BN <= kTpMaxNeurons && tp_smem_bytes(c.T, c.K, true) <= kTpMaxSmem;
     // blocks of the forward and backward kernels that fit on one SM. The backward's is taken
     // for the build without dL/dbeta, so that both builds of a layer share one tiling (and sum
@@ -336,6 +370,40 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
     if (pl->keep_vs) pl->saved_bytes = (size_t)c.T * (size_t)BN * sizeof(float);
     pl->saved_bytes = (pl->saved_bytes + 15) / 16 * 16;
     return DENDSN_OK;
+}
+
+// The plan of a configuration: a pure function of its fields and the current device, which costs
+// several microseconds (the tiling search and two residency queries), more than the launch it
+// precedes. Each thread keeps the last few it made, by value.
+dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
+    if (cfg == nullptr) return fail(DENDSN_ERR_INVALID_ARG, "cfg is NULL");
+    static_assert(sizeof(dendsn_config) == 18 * 4, "compared as bytes: no padding");
+    struct Kept {
+        dendsn_config cfg;
+        int dev;
+        Plan plan;
+    };
+    constexpr int kKept = 16;
+    static thread_local Kept kept[kKept];
+    static thread_local int n = 0, at = 0;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        dev = -1;                                  // no device: nothing is kept
+    }
+    for (int i = 0; i < n; ++i) {
+        if (kept[i].dev == dev && std::memcmp(&kept[i].cfg, cfg, sizeof *cfg) == 0) {
+            *pl = kept[i].plan;
+            return DENDSN_OK;
+        }
+    }
+    const dendsn_status st = compute_plan(*cfg, pl);
+    if (st == DENDSN_OK && dev >= 0) {
+        kept[at] = Kept{*cfg, dev, *pl};
+        at = (at + 1) % kKept;
+        if (n < kKept) ++n;
+    }
+    return st;
 }
 
 Params make_params(const dendsn_config &c, const float *alpha, const float *xi,
