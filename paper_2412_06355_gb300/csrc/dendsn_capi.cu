@@ -311,10 +311,12 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
     pl->gf = g;
     pl->gb = g;
     const int KTB = bwd_lane_compartments(c.K, c.G, c.x_dtype, g.L);
-    tile_columns(pl->gf, fwd_threads(c.K), c.K / KT);
-    tile_columns(pl->gb, bwd_threads(KTB), c.K / KTB);
     pl->sx = (c.x_dtype == DENDSN_BF16) ? 2 : 4;
     pl->layout = (c.K > 1 && c.inner > 1) ? c.layout : 0;   // otherwise the layouts coincide
+    const int nt_f = takes_chunk_forward(c.T, BN, pl->layout, c.inner, c.K, c.x_dtype) ? kChunkFwdThreads
+                                                                                 : fwd_threads(c.K);
+    tile_columns(pl->gf, nt_f, c.K / KT);
+    tile_columns(pl->gb, bwd_threads(KTB), c.K / KTB);
     // narrow layers with long horizons: one block per neuron, time scanned in parallel
     pl->tp = c.T >= kTpMinT && BN <= kTpMaxNeurons && tp_smem_bytes(c.T, c.K, true) <= kTpMaxSmem;
     // blocks of the forward and backward kernels that fit on one SM. The backward's is taken
@@ -342,7 +344,7 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
             (void)cudaGetLastError();
         }
     }
-    dendsn_status st = tile_rows(pl->gf, sms, res_f, 16, &bf);
+    dendsn_status st = tile_rows(pl->gf, sms, res_f, 16 * 256 / nt_f, &bf);
     if (st != DENDSN_OK) return st;
     // backward without the residency: when every column is its own channel (inner = 1)
     // each thread's parameter setup is heavier, and twice the rows per thread measured

@@ -2446,6 +2446,7 @@ dendsn_backward_rowpair_kernel(const BwdArgs A) {
 }  // namespace dendsn
 
 #include "dendsn_twin.cuh"
+#include "dendsn_chunk.cuh"
 
 namespace dendsn {
 
@@ -2523,6 +2524,12 @@ cudaError_t launch_forward(const FwdArgs &a, int blocks, cudaStream_t s, int *re
     using XI = XIO<T, KT, LAYOUT>;
     constexpr size_t raw = sizeof(typename XI::Raw);
     constexpr int NT = fwd_threads(K);
+    if constexpr (XI::kAsync) {
+        if (takes_chunk_forward(a.g.T, a.g.BN, LAYOUT, a.g.inner, K, XT))
+            return launch_or_query(dendsn_forward_chunk_kernel<K, G, PSI, T, LAYOUT>, a, blocks, kChunkFwdThreads,
+                                   chunk_fwd_bytes<typename XI::Raw>(kChunkFwdThreads) +
+                                       kappa_smem_bytes(a.p.mask_mode, KT / G, kChunkFwdThreads), s, resident);
+    }
     if constexpr (LAYOUT == 1 && K == 8 && XT == 0) {
         // 8 float32 compartments, warps of 32 consecutive positions: staged per warp in 16-byte
         // copies; the twin forward's 8-byte ones measured slower (T = 64, G = 2, 524288 neurons:

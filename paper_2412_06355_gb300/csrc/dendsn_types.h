@@ -48,9 +48,20 @@ constexpr bool takes_phased_backward(int K, int G, int KT_bwd, int layout, int T
                                      bool residual) {
     return K == 8 && G == 1 && KT_bwd == 8 && layout == 0 && T == L && !residual;
 }
-// Threads per block: the forward always 256; the backward 128 when a lane owns 8
+// Threads per block: the forward 256 (128 in chunks, below); the backward 128 when a lane owns 8
 // compartments (its ~165 registers allow three 128-thread blocks per SM).
 constexpr int fwd_threads(int K) { return 256; }
+// Whether the forward walks chunks of 8 steps (dendsn_chunk.cuh): rows of more than 8 steps, but
+// for what the twin kernels take (the paper layout with an even H*W), elements of 2 bytes, which
+// cp.async cannot copy, and large float32 layers that stream at the copy rate either way: 8
+// compartments a lane, whose 96 KB of chunks per block leave two blocks per SM, from 262144
+// neurons (T = 12, 4.8M neurons with masks: 335 -> 344 us; T = 1000, 24000 neurons 430 -> 203),
+// and 4 compartments from 2M (T = 64, 4.2M neurons 851 -> 854; T = 32, 2.1M neurons 218 -> 209).
+constexpr int kChunkFwdThreads = 128;
+constexpr bool takes_chunk_forward(int T, int64_t BN, int layout, int inner, int K, int xt) {
+    return T > 8 && (layout == 0 ? K > 1 || xt == 0 : inner % 2 == 1 && xt == 0) &&
+           !(xt == 0 && K >= 4 && BN > (K >= 8 ? 262144 : 2097152));
+}
 constexpr int bwd_threads(int KT) { return KT >= 8 ? 128 : 256; }
 
 // Tiling and sizes shared by every kernel of one call (computed on the host).
