@@ -185,6 +185,10 @@ int sm_count() {
     return cached;
 }
 
+// Capacity of dendsn_backward_noalloc's built-in scratch buffer. Every GPU that loads the library
+// keeps this much device memory reserved until the process exits.
+constexpr size_t kNoAllocScratchBytes = size_t(8) << 20;   // 8 MiB
+
 bool is01(int32_t v) { return v == 0 || v == 1; }
 
 // Column tiling of the O x P neuron matrix for blocks of nt threads with lpn lanes per
@@ -324,13 +328,13 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
     // the parameter gradients in the same order); the two layouts of a layer share it only
     // while a thread has one row (the paper layout's twin kernels fit other block counts).
     int res_f = 0, res_b = 0;
+    BwdArgs ba;
+    std::memset(&ba, 0, sizeof ba);
     if (!pl->tp && O > 0 && c.T > 0) {
         FwdArgs fa;
         std::memset(&fa, 0, sizeof fa);
         fa.g = pl->gf;
         fa.p.mask_mode = c.mask_per_neuron ? 2 : 0;
-        BwdArgs ba;
-        std::memset(&ba, 0, sizeof ba);
         ba.g = pl->gb;
         ba.p.mask_mode = fa.p.mask_mode;
         ba.p.residual = c.residual;
@@ -351,11 +355,23 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
     // faster (token layer 285 -> 272 us); elsewhere 16 blocks per SM measured best
     const int bwd_per_sm = (c.inner == 1) ? 8 : 16;
     if ((st = tile_rows(pl->gb, sms, res_b, bwd_per_sm, &bb)) != DENDSN_OK) return st;
+    const size_t NP = 2 * (size_t)c.K + 2 * (size_t)g.Kb + 1;     // + the beta slot
+    auto scratch_for = [&](int64_t blocks) {
+        return ((size_t)blocks * pl->gb.nch_max * NP * sizeof(float) + 15) / 16 * 16;
+    };
+    pl->scratch_bytes = scratch_for(bb);
+    if (pl->layout == 1 && res_b > 0 && pl->scratch_bytes > kNoAllocScratchBytes) {
+        // the paper layout's own residency may choose more blocks than the compartments-innermost
+        // build's: that one's tiling where the partials would outgrow the built-in buffer
+        if (dispatch_backward(c, 0, g.L, ba, 0, nullptr, &res_b) != cudaSuccess) {
+            res_b = 0;
+            (void)cudaGetLastError();
+        }
+        if ((st = tile_rows(pl->gb, sms, res_b, bwd_per_sm, &bb)) != DENDSN_OK) return st;
+        pl->scratch_bytes = scratch_for(bb);
+    }
     pl->blocks_f = (int)bf;
     pl->blocks_b = (int)bb;
-    const size_t NP = 2 * (size_t)c.K + 2 * (size_t)g.Kb + 1;     // + the beta slot
-    pl->scratch_bytes = (size_t)bb * pl->gb.nch_max * NP * sizeof(float);
-    pl->scratch_bytes = (pl->scratch_bytes + 15) / 16 * 16;
     if (pl->tp) {
         pl->gf.n_ck = pl->gb.n_ck = 0;                 // the backward recomputes from x alone
         pl->scratch_bytes = ((size_t)BN * NP * sizeof(float) + 15) / 16 * 16;
@@ -671,9 +687,6 @@ uint64_t dendsn_launch_count(void) { return g_launches.load(std::memory_order_re
 // fixed buffer compiled into the library instead of caller memory.
 namespace {
 
-// Capacity of the built-in scratch buffer. Every GPU that loads the library keeps this
-// much device memory reserved until the process exits.
-constexpr size_t kNoAllocScratchBytes = size_t(8) << 20;   // 8 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
 constexpr int kMaxDevices = 256;

@@ -13,7 +13,8 @@
 // registers (the backward of rows of at most 4 steps). In the paper's (C_o, P, H, W)
 // layout a lane's compartments are H*W apart; when H*W is even most layers take the twin
 // kernels (dendsn_twin.cuh: two neighbouring neurons per thread), and the forward of 8
-// float32 compartments stages each warp's inputs together (dendsn_forward_staged_kernel).
+// float32 compartments stages each warp's inputs together (dendsn_forward_staged_kernel). The
+// forward of rows of more than 8 steps mostly walks chunks (dendsn_chunk.cuh).
 //
 // Forward (Eqs. methods-compartment .. methods-lif-fire): V^d, V^s and S stay in
 // registers across all T steps; the HBM traffic per step is the K inputs read and

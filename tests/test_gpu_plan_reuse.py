@@ -44,3 +44,16 @@ def test_values_decide():
     cfg.K = 3
     with pytest.raises(binding.DendSNError):
         binding.dendsn_workspace_size(cfg)
+
+
+def test_paper_layout_scratch_stays_within_the_built_in_buffer():
+    """The paper layout is tiled by its own kernels' residency; where the compartments-innermost
+    layer fits the 8 MiB buffer of dendsn_backward_noalloc, so does the paper one."""
+    torch.zeros(1, device="cuda")
+    for K in (2, 8, 16):
+        for C, inner in ((2048, 2), (1024, 4), (512, 16), (64, 256)):
+            for B in (64, 512):
+                for T in (4, 6, 8, 16):
+                    a, b = (binding.dendsn_workspace_size(binding.make_config(
+                        T, B, C * inner, K, 1, C, inner, layout=lay))[1] for lay in ("kinner", "paper"))
+                    assert b <= max(a, 8 << 20), (K, C, inner, B, T)
