@@ -11,7 +11,7 @@
 //
 // What bounds them, and what they measured on GB300 (us before -> after): bfloat16 layers move
 // half the bytes and are bound by instruction issue: T = 6, K = 4, G = 2, B = 128, 128 x 32 x 32
-// backward 1330 -> 467 (266 instructions per pair and step from 357 in a first version that let
+// backward 1330 -> 467 (242 instructions per pair and step from 357 in a first version that let
 // the compiler rebuild every parameter pair and tested every step's bounds; floating-point pipe
 // half busy, memory floor 272), forward 297 -> 189 (floor 151). Float32 layers come close to
 // memory: T = 4, K = 4, G = 2, B = 64, 128 x 32 x 32 backward 224 -> 193 (floor 181).
