@@ -363,7 +363,9 @@ __device__ __forceinline__ void tp_soma_run(const TpGeom &q, float beta, float t
 }
 
 // Below 512 steps the whole horizon costs no more than a guess and its rounds: Z in plain step
-// order in vs, replaced by V^s, serially (every lane of the warp the same).
+// order in vs, replaced by V^s, serially. One thread runs it: it reads Z two vectors ahead of the
+// words it overwrites, so a second thread running the same loop could find V^s where it expects Z
+// (nothing orders the lanes of a warp). The barrier after it publishes V^s.
 template <bool SOFT>
 __device__ __forceinline__ void tp_soma_serial(int T, float beta, float theta, float *vs) {
     float v = SOFT && theta <= 0.f ? theta : 0.f;      // see tp_soma_run
@@ -413,14 +415,14 @@ __device__ __forceinline__ void tp_forward_pass(const Params &P, const TpGeom &q
         else zs[slot] = z;
     });
     __syncthreads();
-    if (w == 0) {
-        if (q.serial()) {
+    if (q.serial()) {
+        if (threadIdx.x == 0) {
             if (P.soft) tp_soma_serial<true>(q.T, P.beta, P.theta, vs);
             else tp_soma_serial<false>(q.T, P.beta, P.theta, vs);
-        } else {
-            if (P.soft) tp_soma_run<true>(q, P.beta, P.theta, zs, vs);
-            else tp_soma_run<false>(q, P.beta, P.theta, zs, vs);
         }
+    } else if (w == 0) {
+        if (P.soft) tp_soma_run<true>(q, P.beta, P.theta, zs, vs);
+        else tp_soma_run<false>(q, P.beta, P.theta, zs, vs);
     }
     __syncthreads();
 }
