@@ -346,7 +346,10 @@ __device__ __forceinline__ void tp_soma_run(const TpGeom &q, float beta, float t
         const unsigned left = __ballot_sync(0xffffffffu, again);
         if (left == 0u) return;
         if (round == kTpRounds) {
-            // the first lane left onwards, by all lanes together
+            // the first lane left onwards, by all lanes together: they rewrite columns that their
+            // own lanes wrote in the rounds before, so those writes have to come first (a vote
+            // or a shuffle orders no memory)
+            __syncwarp();
             const int f = __ffs(left) - 1;
             float cur = __shfl_sync(0xffffffffu, end, f - 1);
             for (int r = f; r < 32; ++r) {

@@ -57,3 +57,11 @@ def check(T, reset, beta, mean, std, N):
 @pytest.mark.parametrize("N", [3, 1001])
 def test_serial_soma(T, reset, beta, mean, std, N):
     check(T, reset, beta, mean, std, N)
+
+
+# whole and ragged segments; guesses that meet, meet late and never meet (the last pass)
+@pytest.mark.parametrize("T", [512, 513, 1000, 2048])
+@pytest.mark.parametrize("reset,beta,mean,std", [("hard", 0.5, 0.3, 1.0), ("hard", 1.0, 0.0, 0.02),
+                                                 ("soft", 1.0, 0.3, 1.0), ("soft", 1.0, 0.0, 0.02)])
+def test_segments(T, reset, beta, mean, std):
+    check(T, reset, beta, mean, std, 9)
