@@ -268,7 +268,9 @@ cudaError_t dispatch_forward(const dendsn_config &cfg, int layout, const FwdArgs
 cudaError_t dispatch_backward(const dendsn_config &cfg, int layout, int L, const BwdArgs &a,
                               int blocks, cudaStream_t s, int *resident = nullptr);
 
-dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
+// *sized: false when a residency query failed, so that the tiling is not by the kernels' residency.
+dendsn_status compute_plan(const dendsn_config &c, Plan *pl, bool *sized) {
+    *sized = true;
     if (c.T < 0 || c.B < 0 || c.N < 0)
         return fail(DENDSN_ERR_INVALID_ARG, "negative size (T=%d B=%d N=%d)", c.T, c.B, c.N);
     if (c.C < 1 || c.inner < 1) return fail(DENDSN_ERR_INVALID_ARG, "C and inner must be >= 1");
@@ -341,10 +343,12 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
         // a failed query (no device) leaves the residency unknown: the fixed sizing applies
         if (dispatch_forward(c, pl->layout, fa, 0, nullptr, &res_f) != cudaSuccess) {
             res_f = 0;
+            *sized = false;
             (void)cudaGetLastError();
         }
         if (dispatch_backward(c, pl->layout, g.L, ba, 0, nullptr, &res_b) != cudaSuccess) {
             res_b = 0;
+            *sized = false;
             (void)cudaGetLastError();
         }
     }
@@ -365,6 +369,7 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
         // build's: that one's tiling where the partials would outgrow the built-in buffer
         if (dispatch_backward(c, 0, g.L, ba, 0, nullptr, &res_b) != cudaSuccess) {
             res_b = 0;
+            *sized = false;
             (void)cudaGetLastError();
         }
         if ((st = tile_rows(pl->gb, sms, res_b, bwd_per_sm, &bb)) != DENDSN_OK) return st;
@@ -390,9 +395,11 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl) {
     return DENDSN_OK;
 }
 
-// The plan of a configuration: a pure function of its fields and the current device, which costs
+// The plan of a configuration: a function of its fields and the current device, which costs
 // several microseconds (the tiling search and two residency queries), more than the launch it
-// precedes. Each thread keeps the last few it made, by value.
+// precedes. Each thread keeps the last few it made, by value; not one whose residency queries
+// failed: its tiling, and with it the scratch it needs, is not the one that another thread (the
+// backward's, say) computes once they succeed.
 dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
     if (cfg == nullptr) return fail(DENDSN_ERR_INVALID_ARG, "cfg is NULL");
     static_assert(sizeof(dendsn_config) == 18 * 4, "compared as bytes: no padding");
@@ -415,8 +422,9 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
             return DENDSN_OK;
         }
     }
-    const dendsn_status st = compute_plan(*cfg, pl);
-    if (st == DENDSN_OK && dev >= 0) {
+    bool sized = false;
+    const dendsn_status st = compute_plan(*cfg, pl, &sized);
+    if (st == DENDSN_OK && sized && dev >= 0) {
         kept[at] = Kept{*cfg, dev, *pl};
         at = (at + 1) % kKept;
         if (n < kKept) ++n;
