@@ -69,7 +69,8 @@ struct TpParams {
             for (int h = 0; h < (Kb < 8 ? 1 : Kb / 8); ++h) m[h] = fetch_mask<(Kb < 8 ? Kb : 8)>(p + 8 * h);
         }
     }
-    // ... and forms what the steps use (load_param_arrays' and apply_neuron_mask's operations).
+    // ... and forms what the steps use (load_param_arrays' and apply_neuron_mask's operations: a
+    // per-neuron mask selects, so that a masked branch's kappa plays no part, whatever its value).
     __device__ __forceinline__ void form(const Params &P) {
         constexpr int MB = Kb < 8 ? Kb : 8;
 #pragma unroll
@@ -89,7 +90,8 @@ struct TpParams {
             }
         }
 #pragma unroll
-        for (int b = 0; b < Kb; ++b) km[b] = __fmul_rn(kap[b], mk[b]);
+        for (int b = 0; b < Kb; ++b)
+            km[b] = P.mask_mode == 2 ? (mk[b] != 0.f ? kap[b] : 0.f) : __fmul_rn(kap[b], mk[b]);
     }
 };
 
