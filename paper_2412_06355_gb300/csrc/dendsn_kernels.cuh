@@ -2452,13 +2452,14 @@ dendsn_backward_rowpair_kernel(const BwdArgs A) {
 namespace dendsn {
 
 // ---------------------------------------------------------------- launchers
-// Dynamic shared memory above 48 KB needs an explicit opt-in per kernel: for as much as a block
-// can have, on the kernel's first launch on a device (an opt-in for each launch's own bytes
-// cost every launch a driver call, and let two threads lower each other's).
+// Shared memory above 48 KB, a kernel's static arrays included, needs an explicit opt-in per kernel:
+// for as much as a block can have, on the kernel's first launch on a device (an opt-in for each
+// launch's own bytes cost every launch a driver call, and let two threads lower each other's).
 cudaError_t allow_all_smem(const void *kernel);
+constexpr size_t kMaxStaticSmem = 1024;            // bytes of static shared memory a kernel may declare
 template <typename Kern>
 cudaError_t allow_smem(Kern kernel, size_t bytes) {
-    return bytes <= 48 * 1024 ? cudaSuccess : allow_all_smem(reinterpret_cast<const void *>(kernel));
+    return bytes + kMaxStaticSmem <= 48 * 1024 ? cudaSuccess : allow_all_smem(reinterpret_cast<const void *>(kernel));
 }
 
 // Blocks of `kernel` (threads, bytes of dynamic shared memory) that fit on one SM, cached

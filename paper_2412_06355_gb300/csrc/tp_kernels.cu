@@ -498,6 +498,7 @@ __global__ void __launch_bounds__(kTpMaxThreads) tp_backward_kernel(const BwdArg
     float *const dz = gsb + q.plane;                   // k2, then dL/dZ
     float *const gvb = dz + q.plane;                   // dL/dV^s (when given)
     __shared__ float red[(kTpMaxThreads / 32) * (2 * KG + 2 * KGb)];
+    static_assert(sizeof red <= kMaxStaticSmem, "allow_smem counts on it");
     const bool has_gv = A.gv != nullptr;
     TpParams<K, G> par;
     par.fetch(P, g, q.n, q.chan);
