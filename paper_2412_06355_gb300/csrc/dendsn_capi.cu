@@ -83,27 +83,29 @@ SmemKey g_smem_done[1024];
 int g_smem_n = 0;
 }  // namespace
 
-// Opts `kernel` in to all the dynamic shared memory a block can have, once per device.
-cudaError_t allow_all_smem(const void *kernel) {
+// Opts `kernel` in to all the dynamic shared memory a block can have, once per device; `again`:
+// whatever is remembered.
+cudaError_t allow_all_smem(const void *kernel, bool again) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     // what this thread saw last, so that the usual call takes no lock
     static thread_local SmemKey seen[64];
     SmemKey &s = seen[(reinterpret_cast<uintptr_t>(kernel) >> 4) % 64];
-    if (s.kernel == kernel && s.device == dev) return cudaSuccess;
+    if (s.kernel == kernel && s.device == dev && !again) return cudaSuccess;
     std::lock_guard<std::mutex> lock(g_smem_mutex);
     bool done = false;
     for (int i = 0; i < g_smem_n && !done; ++i)
         done = g_smem_done[i].kernel == kernel && g_smem_done[i].device == dev;
-    if (!done) {
+    if (!done || again) {
         int most = 0;
         cudaFuncAttributes at;
         if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
         if ((e = cudaFuncGetAttributes(&at, kernel)) != cudaSuccess) return e;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes);
         if (e != cudaSuccess) return e;
-        if (g_smem_n < (int)(sizeof g_smem_done / sizeof g_smem_done[0])) g_smem_done[g_smem_n++] = SmemKey{kernel, dev};
+        if (!done && g_smem_n < (int)(sizeof g_smem_done / sizeof g_smem_done[0]))
+            g_smem_done[g_smem_n++] = SmemKey{kernel, dev};
     }
     s = SmemKey{kernel, dev};
     return cudaSuccess;
@@ -135,7 +137,10 @@ cudaError_t resident_blocks(const void *kernel, int threads, size_t bytes, int *
         }
     }
     int n = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, bytes);
+    e = with_opt_in(kernel, bytes, [&] {
+        const cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, bytes);
+        return q == cudaSuccess && n == 0 ? cudaErrorInvalidValue : q;
+    });
     if (e != cudaSuccess) return e;
     if (g_resident_n < (int)(sizeof g_resident / sizeof g_resident[0]))
         g_resident[g_resident_n++] = ResidentKey{kernel, threads, bytes, dev, n};

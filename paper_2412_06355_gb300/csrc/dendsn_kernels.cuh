@@ -2452,14 +2452,9 @@ dendsn_backward_rowpair_kernel(const BwdArgs A) {
 namespace dendsn {
 
 // ---------------------------------------------------------------- launchers
-// Shared memory above 48 KB, a kernel's static arrays included, needs an explicit opt-in per kernel:
-// for as much as a block can have, on the kernel's first launch on a device (an opt-in for each
-// launch's own bytes cost every launch a driver call, and let two threads lower each other's).
-cudaError_t allow_all_smem(const void *kernel);
-constexpr size_t kMaxStaticSmem = 1024;            // bytes of static shared memory a kernel may declare
 template <typename Kern>
 cudaError_t allow_smem(Kern kernel, size_t bytes) {
-    return bytes + kMaxStaticSmem <= 48 * 1024 ? cudaSuccess : allow_all_smem(reinterpret_cast<const void *>(kernel));
+    return needs_opt_in(bytes) ? allow_all_smem(reinterpret_cast<const void *>(kernel)) : cudaSuccess;
 }
 
 // Blocks of `kernel` (threads, bytes of dynamic shared memory) that fit on one SM, cached
@@ -2485,10 +2480,13 @@ cudaError_t launch_or_query(Kern kernel, const Args &a, int blocks, int threads,
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    return with_opt_in(reinterpret_cast<const void *>(kernel), bytes,
+                       [&] { return cudaLaunchKernelEx(&cfg, kernel, a); });
 #else
-    kernel<<<blocks, threads, bytes, s>>>(a);
-    return cudaGetLastError();
+    return with_opt_in(reinterpret_cast<const void *>(kernel), bytes, [&] {
+        kernel<<<blocks, threads, bytes, s>>>(a);
+        return cudaGetLastError();
+    });
 #endif
 }
 

@@ -123,6 +123,23 @@ struct FinArgs {
     int32_t stateless;
 };
 
+// Shared memory above 48 KB, a kernel's static arrays included, needs an explicit opt-in per kernel:
+// for as much as a block can have, on the kernel's first launch on a device (an opt-in for each
+// launch's own bytes cost every launch a driver call, and let two threads lower each other's).
+cudaError_t allow_all_smem(const void *kernel, bool again = false);
+constexpr size_t kMaxStaticSmem = 1024;            // bytes of static shared memory a kernel may declare
+constexpr bool needs_opt_in(size_t bytes) { return bytes + kMaxStaticSmem > 48 * 1024; }
+// f, which launches or queries `kernel` with `bytes` of dynamic shared memory; when that is refused
+// to a kernel that needs the opt-in, once more after opting in again: an opt-in belongs to a
+// context, and cudaDeviceReset or another driver context of the device brings a new one.
+template <typename F>
+cudaError_t with_opt_in(const void *kernel, size_t bytes, F f) {
+    const cudaError_t e = f();
+    if (e == cudaSuccess || !needs_opt_in(bytes)) return e;
+    (void)cudaGetLastError();
+    return allow_all_smem(kernel, true) == cudaSuccess ? f() : e;
+}
+
 // XT: 0 = float, 1 = bfloat16. LAYOUT: 0 = compartments innermost, 1 = the paper's
 // (C_o, P, H, W) layer layout. Defined in the instantiation units. With `resident` non-null
 // nothing is launched: *resident receives how many blocks of the kernel this call would

@@ -686,7 +686,8 @@ cudaError_t tp_launch(void (*kernel)(Par...), unsigned blocks, unsigned threads,
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = DENDSN_PDL ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, arg...);
+    return with_opt_in(reinterpret_cast<const void *>(kernel), smem,
+                       [&] { return cudaLaunchKernelEx(&cfg, kernel, arg...); });
 }
 
 }  // namespace
