@@ -491,9 +491,11 @@ dendsn_backward_twin_kernel(const BwdArgs A) {
         for (int i = 0; i < KT; ++i) { put(i, a[i]); put(KT + i, nxi[i]); }
 #pragma unroll
         for (int b = 0; b < KTb; ++b) {
+            // a channel's kappa m is a product, in the forward too: NaN for a kappa that is not finite
+            const bool nan = km[b] != km[b];
             put(2 * KT + b, iz[b]);
-            put(2 * KT + KTb + b, kap[b]);
-            if (mk[b] == 0.f) { mb1 &= ~(1u << b); mb2 &= ~(1u << b); }
+            put(2 * KT + KTb + b, nan ? km[b] : kap[b]);
+            if (mk[b] == 0.f && !nan) { mb1 &= ~(1u << b); mb2 &= ~(1u << b); }
         }
     }
 #pragma unroll 1

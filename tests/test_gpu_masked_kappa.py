@@ -38,3 +38,25 @@ def test_a_per_neuron_mask_leaves_the_branch_out(T, bad):
     a, b = run(w, inp), run(w, zero)
     for k in a:
         assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("T", [4, 6, 10])
+@pytest.mark.parametrize("K,G", [(4, 1), (4, 2)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_a_channel_mask_is_the_same_in_both_layouts(T, K, G, dtype):
+    """A channel's kappa m is a product, in the forward and in the backward, whichever kernels run:
+    with an infinite kappa the masked channel's potentials and gradients are NaN, the others' not."""
+    w = workloads.Workload("mk", T=T, B=3, N=102, K=K, G=G, C=3, inner=34, dtype=dtype, psi="mh",
+                           reset="hard", mask_p=0.5, seed=T)
+    out = []
+    for layout in ("paper", "kinner"):
+        inp = to_dev(workloads.make_inputs(w.with_(layout=layout), "cpu"))
+        inp["mask"][:] = 1
+        inp["mask"][1, 0] = 0
+        inp["kappa"][1, 0] = float("inf")
+        out.append(run(w.with_(layout=layout), inp))
+    a, b = out
+    for k in a:
+        x = workloads.from_paper_layout(a[k], w.N, w.K, w.inner) if k == "gx" else a[k]
+        assert torch.equal(x.isnan(), b[k].isnan()) and torch.equal(x.nan_to_num(), b[k].nan_to_num()), k
+    assert a["gx"].isnan().any() and not a["gx"].isnan().all()
