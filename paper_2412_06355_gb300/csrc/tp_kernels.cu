@@ -128,11 +128,17 @@ __device__ __forceinline__ float tp_soma_input(const TpParams<K, G> &q, const fl
     return z;
 }
 
+// Below these many steps the soma runs serially: that costs about what guesses that meet do, and half
+// of what guesses that never meet do (K = 1, one neuron, forward, us, serial / meet / never: T = 512 6.0 /
+// 6.6 / 13, T = 640 7 / 7 / 15, T = 700 8 / 7.4 / 17, T = 1000 11 / 8 / 21).
+constexpr int kTpSerial = 704;
+
 // The neuron's place in x and the horizon's segments. Step t = l * TB + s of segment l sits at
 // slot s * 32 + l of a plane of `plane` floats.
 struct TpGeom {
     int64_t j, n, xo, sX, ks;
     int chan, T, TB, plane;
+    bool plain = false;                          // set by tp_forward_pass
     __device__ __forceinline__ TpGeom(const Geometry &g, int layout) {
         j = blockIdx.x;
         n = j % g.N;
@@ -150,9 +156,9 @@ struct TpGeom {
             ks = g.inner;
         }
     }
-    // V^s of short horizons is in plain step order (tp_soma_serial)
-    __device__ __forceinline__ bool serial() const { return T < 512; }
-    __device__ __forceinline__ int v_at(int slot, int t) const { return serial() ? t : slot; }
+    // V^s of a serial soma is in plain step order
+    __device__ __forceinline__ bool serial() const { return T < kTpSerial; }
+    __device__ __forceinline__ int v_at(int slot, int t) const { return plain ? t : slot; }
     __device__ __forceinline__ int len(int l) const { return max(0, min(TB, T - l * TB)); }
     // f(slot, t) for every step, the block's threads sharing them; consecutive threads take
     // consecutive segments
@@ -306,6 +312,28 @@ __device__ __forceinline__ float tp_charge(float z, float v, float beta, float t
     return __fmaf_rn(tp_keep(v, theta), __fmul_rn(beta, v), z);
 }
 
+// The soma serially: Z in plain step order in vs, replaced by V^s. Below kTpSerial steps the whole
+// horizon costs no more this way than a guess and its rounds. One thread runs it: it reads Z two vectors ahead of the
+// words it overwrites, so a second thread running the same loop could find V^s where it expects Z
+// (nothing orders the lanes of a warp). The barrier after it publishes V^s.
+template <bool SOFT>
+__device__ __forceinline__ void tp_soma_serial(int T, float beta, float theta, float *vs) {
+    float v = SOFT && theta <= 0.f ? theta : 0.f;      // the state before a first step (tp_soma_run)
+    float4 *p = reinterpret_cast<float4 *>(vs);        // planes hold a whole number of 32 steps
+    float4 a = p[0], b = p[1];
+    for (int t = 0; t < T; t += 8, p += 2) {
+        const bool more = t + 8 < T;
+        const float4 na = more ? p[2] : a, nb = more ? p[3] : b;
+        float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int u = 0; u < 8; ++u) z[u] = v = tp_charge<SOFT>(z[u], v, beta, theta);
+        p[0] = make_float4(z[0], z[1], z[2], z[3]);
+        p[1] = make_float4(z[4], z[5], z[6], z[7]);
+        a = na;
+        b = nb;
+    }
+}
+
 // Soma over Z[t] (zs), V^s[t] to vs, by one warp. The recursion is not linear, but trajectories
 // from different states soon coincide exactly (a spike's reset forgets the state; the leak
 // shrinks a difference until it rounds away). So every lane guesses the state entering its
@@ -313,12 +341,17 @@ __device__ __forceinline__ float tp_charge(float z, float v, float beta, float t
 // its own. The lane before it ends in the state that should have been guessed: lanes whose guess
 // is not that state, bit for bit, run their segment again from it, for a few rounds (segment 0 is
 // exact, so after round r segments 0 .. r are); what still differs then is run segment after
-// segment. What is kept is always the serial recursion's own operations on its own values. The
-// usual cost is the guess and a segment or two instead of the horizon; the worst case (guesses
-// that never meet, e.g. a soft reset with beta near 1) repeats the serial work.
-constexpr int kTpGuess = 192, kTpRounds = 4;
+// segment, or, when that is more than a few, the horizon serially in plain step order (then the
+// result is true, and vs in that order). What is kept is always the serial recursion's own
+// operations on its own values. The usual cost is the guess and a segment or two instead of the
+// horizon; the worst case (guesses that never meet, e.g. a soft reset with beta near 1) adds the
+// serial work. Forward, K = 4, G = 2, us: one neuron of 2048 steps 10 when guesses meet and 31 when they
+// never do (36 with the segments one after the other), of 2400 steps 12 and 36 (44), 2048 neurons of
+// 2400 steps 117 and 238 (279).
+constexpr int kTpGuess = 192, kTpRounds = 4, kTpFew = 12;
+
 template <bool SOFT>
-__device__ __forceinline__ void tp_soma_run(const TpGeom &q, float beta, float theta, const float *zs, float *vs) {
+__device__ __forceinline__ bool tp_soma_run(const TpGeom &q, float beta, float theta, const float *zs, float *vs) {
     const int l = threadIdx.x & 31;
     const int n = q.len(l);
     // segment r (n_r steps) from the state `start`, V^s to vs; returns its last state
@@ -346,46 +379,36 @@ __device__ __forceinline__ void tp_soma_run(const TpGeom &q, float beta, float t
         const float before = __shfl_up_sync(0xffffffffu, end, 1);
         const bool again = l > 0 && n > 0 && __float_as_int(before) != __float_as_int(start);
         const unsigned left = __ballot_sync(0xffffffffu, again);
-        if (left == 0u) return;
+        if (left == 0u) return false;
         if (round == kTpRounds) {
-            // the first lane left onwards, by all lanes together: they rewrite columns that their
-            // own lanes wrote in the rounds before, so those writes have to come first (a vote
-            // or a shuffle orders no memory)
+            // both ways rewrite columns that their own lanes wrote in the rounds before, so those
+            // writes have to come first (a vote or a shuffle orders no memory)
             __syncwarp();
+            if (__popc(left) > kTpFew) {
+                // an even TB would put the lanes' words in the same banks: every lane starts elsewhere
+                const int first = q.TB % 2 == 0 ? l % q.TB : 0;
+#pragma unroll 4
+                for (int i = 0; i < q.TB; ++i) {
+                    const int s = i + first < q.TB ? i + first : i + first - q.TB;
+                    if (s < n) vs[l * q.TB + s] = zs[s * 32 + l];
+                }
+                __syncwarp();
+                if (l == 0) tp_soma_serial<SOFT>(q.T, beta, theta, vs);
+                return true;
+            }
+            // the first lane left onwards, by all lanes together
             const int f = __ffs(left) - 1;
             float cur = __shfl_sync(0xffffffffu, end, f - 1);
             for (int r = f; r < 32; ++r) {
                 const float st = __shfl_sync(0xffffffffu, start, r), en = __shfl_sync(0xffffffffu, end, r);
                 cur = __float_as_int(cur) == __float_as_int(st) ? en : segment(r, q.len(r), cur);
             }
-            return;
+            return false;
         }
         if (again) {
             start = before;
             end = segment(l, n, start);
         }
-    }
-}
-
-// Below 512 steps the whole horizon costs no more than a guess and its rounds: Z in plain step
-// order in vs, replaced by V^s, serially. One thread runs it: it reads Z two vectors ahead of the
-// words it overwrites, so a second thread running the same loop could find V^s where it expects Z
-// (nothing orders the lanes of a warp). The barrier after it publishes V^s.
-template <bool SOFT>
-__device__ __forceinline__ void tp_soma_serial(int T, float beta, float theta, float *vs) {
-    float v = SOFT && theta <= 0.f ? theta : 0.f;      // see tp_soma_run
-    float4 *p = reinterpret_cast<float4 *>(vs);        // planes hold a whole number of 32 steps
-    float4 a = p[0], b = p[1];
-    for (int t = 0; t < T; t += 8, p += 2) {
-        const bool more = t + 8 < T;
-        const float4 na = more ? p[2] : a, nb = more ? p[3] : b;
-        float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int u = 0; u < 8; ++u) z[u] = v = tp_charge<SOFT>(z[u], v, beta, theta);
-        p[0] = make_float4(z[0], z[1], z[2], z[3]);
-        p[1] = make_float4(z[4], z[5], z[6], z[7]);
-        a = na;
-        b = nb;
     }
 }
 
@@ -398,7 +421,7 @@ __device__ __forceinline__ float tp_alpha(const Params &P, const TpGeom &q) {
 
 // V^d over x in the planes xv, Z in zs, V^s in vs (zs holds the residual sums on entry).
 template <int K, int G>
-__device__ __forceinline__ void tp_forward_pass(const Params &P, const TpGeom &q, const TpParams<K, G> &par,
+__device__ __forceinline__ void tp_forward_pass(const Params &P, TpGeom &q, const TpParams<K, G> &par,
                                                 float alpha, int psi, float *xv, float *zs, float *vs) {
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const bool residual = P.residual != 0;
@@ -420,16 +443,16 @@ __device__ __forceinline__ void tp_forward_pass(const Params &P, const TpGeom &q
         else zs[slot] = z;
     });
     __syncthreads();
-    if (q.serial()) {
+    bool plain = q.serial();
+    if (plain) {
         if (threadIdx.x == 0) {
             if (P.soft) tp_soma_serial<true>(q.T, P.beta, P.theta, vs);
             else tp_soma_serial<false>(q.T, P.beta, P.theta, vs);
         }
     } else if (w == 0) {
-        if (P.soft) tp_soma_run<true>(q, P.beta, P.theta, zs, vs);
-        else tp_soma_run<false>(q, P.beta, P.theta, zs, vs);
+        plain = P.soft ? tp_soma_run<true>(q, P.beta, P.theta, zs, vs) : tp_soma_run<false>(q, P.beta, P.theta, zs, vs);
     }
-    __syncthreads();
+    q.plain = __syncthreads_or(plain);
 }
 
 template <int K, int G, typename XT>
@@ -437,7 +460,7 @@ __global__ void __launch_bounds__(kTpMaxThreads) tp_forward_kernel(const FwdArgs
     pdl_wait();
     const Geometry &g = A.g;
     const Params &P = A.p;
-    const TpGeom q(g, layout);
+    TpGeom q(g, layout);
     extern __shared__ float tp_smem[];
     float *const xv = tp_smem;                         // [K]: x, then V^d
     float *const zs = xv + K * q.plane;                // Z
@@ -489,7 +512,7 @@ __global__ void __launch_bounds__(kTpMaxThreads) tp_backward_kernel(const BwdArg
     constexpr int KGb = KG / G;
     const Geometry &g = A.g;
     const Params &P = A.p;
-    const TpGeom q(g, layout);
+    TpGeom q(g, layout);
     extern __shared__ float tp_smem[];
     float *const vdh = tp_smem;                        // [K]: x, then V^d
     float *const zsb = vdh + K * q.plane;              // Z, then k1

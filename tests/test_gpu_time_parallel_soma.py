@@ -65,3 +65,21 @@ def test_serial_soma(T, reset, beta, mean, std, N):
                                                  ("soft", 1.0, 0.3, 1.0), ("soft", 1.0, 0.0, 0.02)])
 def test_segments(T, reset, beta, mean, std):
     check(T, reset, beta, mean, std, 9)
+
+
+# the line between the serial loop and the segments, and the last pass: from the first segment on
+# (most guesses never meet) or over the few segments of a quiet stretch
+@pytest.mark.parametrize("T,N,quiet", [(703, 5, 0), (704, 5, 0), (705, 5, 0), (737, 5, 0), (2400, 5, 0), (705, 1001, 0),
+                                       (1000, 5, 300), (2048, 5, 640), (2048, 5, 900)])
+@pytest.mark.parametrize("reset,std", [("hard", 0.02), ("soft", 0.02), ("soft", 1.0)])
+def test_the_last_pass(T, N, quiet, reset, std):
+    w = workloads.Workload("soma", T=T, B=2, N=N, K=4, G=2, C=1, inner=N, dtype="f32", psi="mh",
+                           reset="hard", beta=0.0, x_mean=0.3 if quiet else 0.0, x_std=std, seed=T + N)
+    inp = workloads.make_inputs(w, "cpu")
+    if quiet:
+        inp["x"][T - quiet:] *= 1e-3
+    _, z = potentials(w, inp)
+    s, v = potentials(w.with_(reset=reset, beta=1.0), inp)
+    ref = serial(z, 1.0, w.theta, reset == "soft")
+    assert np.array_equal(v, ref)
+    assert np.array_equal(s, (ref >= np.float32(w.theta)).astype(np.float32))
