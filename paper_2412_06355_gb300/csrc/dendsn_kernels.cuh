@@ -2504,17 +2504,34 @@ inline bool takes_twin(const Geometry &g, const void *a, const void *b, size_t s
 // 29 -> 33).
 template <int G, int PSI, int L>
 constexpr bool twin_backward() { return !(PSI == PSI_IDENTITY && G > 1) && !(G == 4 && L == 8); }
-// Float32 lanes of up to 4 compartments over several chunks: the chunk's buffers, checkpoints and
-// two-level sums leave room for two blocks per SM only (T = 29, K = 4, G = 2, B = 32: 134 ->
-// 139; T = 64 about equal). Lanes of 8 compartments need enough neurons to hide a unit loop
-// that a small layer sees as latency (K = 8, G = 2, float32: T = 127, 8192 neurons 68 -> 78,
-// 32768 neurons 133 -> 116; T = 64, 16384 neurons 34 -> 38, 32768 neurons 53 -> 45), and more
-// of them when much of a row is an incomplete chunk (bfloat16 T = 10: 131072 neurons 35 -> 39,
-// 524288 neurons 144 -> 140; T = 5: 131072 neurons 20 -> 20, 524288 neurons 72 -> 53).
-inline bool twin_pays(const Geometry &g, int KT, bool f32) {
+// Which calls the twin backward takes, for KT compartments a lane (times of the one-neuron kernel,
+// GB300: geometric means over H*W from 8 to 3136, 1 to 1024 channels and all the compiled (K, G) that
+// the line holds for; single layers scatter by 10 to 30% around them with how full their last wave is):
+// - H*W below 8: a block's tile spans so many channels that summing their gradients costs what the
+//   pairs save, or more: K = 4 and 16 on float32 lanes of 4, G = 1, 1.06 to 1.18, 8-compartment lanes
+//   T <= 4 1.0 to 1.46, float32 K = 8 1.01 to 1.26, K = 16, G = 2, T > 8 1.08 to 1.19 (what stays:
+//   0.7 to 1.08).
+// - Float32 lanes of up to 4 compartments over several chunks: the chunk's buffers, checkpoints and
+//   two-level sums leave room for two blocks per SM only (T = 9 to 12, G = 1 1.06 to 1.19, G = 2
+//   0.98 to 1.06).
+// - Lanes of 8, rows of 1 to 3 steps: the parameters' way through shared memory is paid by a few steps, so
+//   it takes many rows per thread. bfloat16 T = 2 262144 lanes 1.2, 524288 1.1, 1M 0.8 to 1.0; T = 3
+//   262144 1.06 to 1.19, 524288 0.85 to 0.99; T = 1 G = 1 1.2 to 1.4 up to 2M and 0.98 at 4M, G = 2 1.07
+//   at 2M and 0.87 at 4M, G = 4 0.97 at 1M; float32 T = 1 G = 2 1.2 everywhere, G = 4 0.99 at 2M.
+// - Lanes of 8, float32, G = 1, T = 9: a second chunk of one step (1.00 to 1.04; T = 10 0.91 to 0.99).
+// - Other lanes of 8: complete chunks from 24576 (T = 8 0.8 to 0.89, T = 16 0.75 to 0.94 between there
+//   and 65536), the others from 131072 (bfloat16, 131072 to 200000: T = 5 0.71 to 0.89, T = 7 0.65 to
+//   0.82, T = 10 0.69 to 0.93; float32 T = 5 0.87 to 0.90, T = 10 0.97).
+inline bool twin_pays(const Geometry &g, int KT, int G, bool f32) {
+    const int64_t lanes = g.BN * (g.K / KT);
+    if (g.inner < 8 && (KT == 8 ? g.T <= 4 || (f32 && (g.K == 8 || (G > 1 && g.T > 8)))
+                                : KT == 4 && f32 && G == 1 && g.K != 8)) return false;
     if (KT < 8) return !(f32 && g.n_ck > 0);
+    if (g.T == 1) return G > (f32 ? 2 : 1) && lanes > (G == 2 ? 2100000 : 1000000);
+    if (!f32 && g.T < 4) return lanes * g.T > 1200000;
+    if (f32 && G == 1 && g.T == 9) return false;
     const bool whole = g.T <= 4 ? g.T == 4 : (g.T == 6 || g.T % 8 == 0 || g.T >= 32);
-    return g.BN * (g.K / KT) > (whole ? 24576 : 131072);
+    return lanes > (whole ? 24576 : 131072);
 }
 
 template <int K, int G, int PSI, int XT, int LAYOUT>
@@ -2606,7 +2623,7 @@ cudaError_t launch_backward(const BwdArgs &a, int blocks, cudaStream_t s, int *r
     }
     // the paper layout with an even H*W: two neighbouring neurons per thread
     if constexpr (LAYOUT == 1 && K >= 2 && twin_backward<G, PSI, L>()) {
-        if (takes_twin(a.g, a.gs, nullptr, sizeof(T), 0) && twin_pays(a.g, KT, XT == 0)) {
+        if (takes_twin(a.g, a.gs, nullptr, sizeof(T), 0) && twin_pays(a.g, KT, G, XT == 0)) {
             constexpr int NTW = NT / 2;
             auto twin = [&](auto lc, auto full) {
                 constexpr int LC = decltype(lc)::value;

@@ -53,14 +53,17 @@ constexpr bool takes_phased_backward(int K, int G, int KT_bwd, int layout, int T
 constexpr int fwd_threads(int K) { return 256; }
 // Whether the forward walks chunks of 8 steps (dendsn_chunk.cuh): rows of more than 8 steps, but
 // for what the twin kernels take (the paper layout with an even H*W), elements of 2 bytes, which
-// cp.async cannot copy, and large float32 layers that stream at the copy rate either way: 8
-// compartments a lane, whose 96 KB of chunks per block leave two blocks per SM, from 262144
-// neurons (T = 12, 4.8M neurons with masks: 335 -> 344 us; T = 1000, 24000 neurons 430 -> 203),
-// and 4 compartments from 2M (T = 64, 4.2M neurons 851 -> 854; T = 32, 2.1M neurons 218 -> 209).
+// cp.async cannot copy, and large float32 layers that stream at the copy rate either way: lanes of
+// 8 compartments, whose 96 KB of chunks per block leave two blocks per SM, with K = 8 above 262144
+// neurons (times of step by step, T = 9 to 64: 16384 neurons 0.57 to 0.83, 98304 0.73 to 0.89, 196608
+// 0.93 to 1.07, 262144 0.91 to 1.07, above 0.93 to 1.02; T = 12, 4.8M with masks 335 -> 344 us), with
+// K = 16, twice the lanes, above 24576 (16384 neurons 0.73 to 1.0, 32768 0.9 to 1.08, 65536 1.0 to 1.14,
+// 131072 0.95 to 1.17), and 4 compartments from 2M (T = 64, 4.2M neurons 851 -> 854; T = 32, 2.1M
+// neurons 218 -> 209).
 constexpr int kChunkFwdThreads = 128;
 constexpr bool takes_chunk_forward(int T, int64_t BN, int layout, int inner, int K, int xt) {
     return T > 8 && (layout == 0 ? K > 1 || xt == 0 : inner % 2 == 1 && xt == 0) &&
-           !(xt == 0 && K >= 4 && BN > (K >= 8 ? 262144 : 2097152));
+           !(xt == 0 && K >= 4 && BN > (K == 16 ? 24576 : K == 8 ? 262144 : 2097152));
 }
 constexpr int bwd_threads(int KT) { return KT >= 8 ? 128 : 256; }
 

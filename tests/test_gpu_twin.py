@@ -104,3 +104,39 @@ def test_against_the_oracle(T, K, G, dtype, B, C, inner, kw):
     w = workloads.Workload("twin8", T=T, B=B, N=C * inner, K=K, G=G, C=C, inner=inner, dtype=dtype,
                            psi="mh", reset="hard", layout="paper", seed=7 * T + K).with_(**kw)
     check_layer(w)
+
+
+# forwards: spikes (by elements) and V^s (by floats) that are not aligned for a pair
+@pytest.mark.parametrize("T,dtype,inner", [(6, "bf16", 34), (10, "bf16", 100), (4, "f32", 6)])
+@pytest.mark.parametrize("spike_offset,v_offset", [(1, 0), (0, 1), (1, 1)])
+def test_element_aligned_outputs_get_the_same_bits(T, dtype, inner, spike_offset, v_offset):
+    w = make(T, 4, 2, dtype, inner, layout="paper")
+    inp = to_dev(workloads.make_inputs(w, "cpu"))
+    cfg = binding.config_of(w)
+    p = [inp[k] for k in ("alpha", "xi", "zeta", "kappa")]
+    s0, v0 = binding.forward(cfg, inp["x"], *p, None, want_v=True)
+    s = torch.empty(s0.numel() + spike_offset, dtype=s0.dtype, device="cuda")[spike_offset:].view(s0.shape)
+    v = torch.empty(v0.numel() + v_offset, device="cuda")[v_offset:].view(v0.shape)
+    binding.dendsn_forward(cfg, inp["x"], *p, None, s, v)
+    assert torch.equal(s, s0) and torch.equal(v, v0)
+
+
+# layers just beyond the sizes from which rows of a few steps take the twin backward: the same bits per neuron as the compartments-innermost layer
+@pytest.mark.parametrize("T,B,K,G,dtype,psi", [
+    (2, 150, 8, 1, "bf16", "mh"), (3, 100, 8, 2, "bf16", "mh"), (1, 600, 8, 2, "bf16", "mh"), (1, 300, 8, 4, "f32", "mh")])
+def test_large_layers_bitwise(T, B, K, G, dtype, psi):
+    w = workloads.Workload("twinl", T=T, B=B, N=4096, K=K, G=G, C=64, inner=64, dtype=dtype, psi=psi,
+                           reset="hard", seed=T)
+    out = []
+    for layout in ("paper", "kinner"):
+        wl = w.with_(layout=layout)
+        inp = workloads.make_inputs(wl, "cuda")
+        cfg = binding.config_of(wl)
+        p = [inp[k] for k in ("alpha", "xi", "zeta", "kappa")]
+        saved, scratch = binding.workspace(cfg)
+        s, v = binding.forward(cfg, inp["x"], *p, None, want_v=True, saved=saved)
+        g = binding.backward(cfg, inp["x"], *p, None, inp["gs"], None, saved, scratch)
+        gx = workloads.from_paper_layout(g["gx"], w.N, w.K, w.inner) if layout == "paper" else g["gx"]
+        out.append((s, v, gx))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)

@@ -1,0 +1,39 @@
+"""Which kernels a layer takes at the lines of the dispatch rules, as the library itself launches them
+on a stand-in for the CUDA runtime (no GPU)."""
+import pytest
+
+from paper_2412_06355_gb300 import binding
+
+from fake_runtime import Library
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return Library(str(tmp_path_factory.mktemp("fake")))
+
+
+TWIN, ONE, SHORT = "dendsn_backward_twin_kernel", "dendsn_backward_kernel", "dendsn_backward_twin_short_kernel"
+
+
+# T, neurons per sample, H*W, samples, K, G, dtype, the backward
+@pytest.mark.parametrize("T,N,inner,B,K,G,dtype,want", [
+    (8, 4096, 64, 6, 8, 1, "bf16", ONE), (8, 4096, 64, 7, 8, 1, "bf16", TWIN),       # 24576 lanes
+    (10, 4096, 64, 32, 8, 1, "bf16", ONE), (10, 4096, 64, 33, 8, 1, "bf16", TWIN),   # 131072
+    (9, 4096, 64, 40, 8, 1, "bf16", TWIN), (9, 4096, 64, 40, 8, 1, "f32", ONE), (9, 4096, 64, 40, 8, 2, "f32", TWIN),
+    (1, 4096, 64, 300, 8, 1, "bf16", ONE), (1, 4096, 64, 300, 8, 2, "bf16", ONE), (1, 4096, 64, 300, 8, 4, "bf16", TWIN),
+    (1, 4096, 64, 600, 8, 2, "bf16", TWIN), (1, 4096, 64, 600, 8, 2, "f32", ONE), (1, 4096, 64, 600, 8, 4, "f32", TWIN),
+    (2, 4096, 64, 140, 8, 1, "bf16", ONE), (2, 4096, 64, 150, 8, 1, "bf16", TWIN), (2, 4096, 64, 40, 8, 2, "f32", TWIN),
+    (3, 4096, 64, 90, 8, 1, "bf16", ONE), (3, 4096, 64, 100, 8, 1, "bf16", TWIN),
+    (4, 4096, 64, 7, 8, 2, "bf16", TWIN), (4, 4096, 64, 6, 8, 2, "bf16", ONE),
+    (4, 4096, 4, 100, 8, 2, "bf16", ONE), (8, 4096, 4, 100, 8, 2, "bf16", TWIN), (8, 4096, 4, 100, 8, 2, "f32", ONE),
+    (8, 4096, 8, 100, 8, 2, "f32", TWIN), (8, 4096, 4, 100, 16, 2, "f32", TWIN),
+    (16, 4096, 4, 100, 16, 2, "f32", ONE), (16, 4096, 4, 100, 16, 1, "f32", TWIN),
+    (4, 4096, 4, 10, 4, 1, "f32", ONE), (4, 4096, 4, 10, 4, 2, "f32", SHORT), (4, 4096, 8, 10, 4, 1, "f32", SHORT),
+    (6, 4096, 64, 10, 4, 1, "f32", TWIN), (9, 4096, 64, 10, 4, 1, "f32", ONE), (9, 4096, 64, 10, 4, 1, "bf16", TWIN),
+])
+def test_the_paper_layouts_backward(fake, T, N, inner, B, K, G, dtype, want):
+    cfg = binding.make_config(T, B, N, K, G, N // inner, inner, dtype, layout="paper")
+    assert fake.launches(cfg)[1] == want
+    # never with dL/dS that is aligned for an element but not for a pair
+    if want == TWIN:
+        assert fake.launches(cfg, gs=(1 << 20) + (2 if dtype == "bf16" else 4))[1] != TWIN
