@@ -1202,8 +1202,8 @@ dendsn_forward_kernel(const FwdArgs A) {
     }
 }
 
-// Forward in the paper's (C_o, P, H, W) layout with the inputs staged per warp. Used for 8
-// float32 compartments when H*W and the column tile are multiples of 32: a
+// Forward in the paper's (C_o, P, H, W) layout with the inputs staged per warp. Used where
+// staged_forward and staged_pays say, when H*W and the column tile are multiples of 32: a
 // warp's 32 neurons are then 32 consecutive positions of one channel group, so compartment k
 // of all of them is one contiguous run of 32 elements. Each lane copies its share of the
 // warp's K runs with 16-byte cp.async into the slot [k][32 lanes] (one copy per lane per
@@ -2534,6 +2534,26 @@ inline bool twin_pays(const Geometry &g, int KT, int G, bool f32) {
     return lanes > (whole ? 24576 : 131072);
 }
 
+// The paper-layout forwards that are staged per warp (warps of 32 consecutive positions, 16-byte
+// copies) rather than run on twins, where they have the choice (us staged -> twin, GB300):
+// - 8 float32 compartments: the twin's 8-byte copies are slower (T = 64, G = 2, 524288 neurons 193 ->
+//   210; T = 6, G = 1, 1M neurons 37.5 -> 39.8).
+// - 4 float32 compartments of one branch once the inputs no longer stay in L2: T = 6, 1M neurons
+//   (100 MB) 21 -> 26, 4M 81 -> 87; T = 32, 327680 neurons (168 MB) 38 -> 47; below, twins (T = 6,
+//   524288 neurons 0.74 times, T = 4, 1M, 67 MB, 0.81 times).
+// - 8 bfloat16 compartments, two per branch, the identity, rows that end in an incomplete chunk of
+//   8 steps: without an exponential the chunk's tests weigh more (T = 17, 16384 neurons 8.3 -> 9.7;
+//   T = 10, 1M neurons 64 -> 72), but for the sizes between, where the twins' smaller blocks fill
+//   their waves better (T = 10, 98304 neurons 0.77 times, 327680 24.5 -> 21.2).
+template <int K, int G, int PSI, int XT>
+constexpr bool staged_forward() {
+    return XT == 0 ? K == 8 || (K == 4 && G == 4) : K == 8 && G == 2 && PSI == PSI_IDENTITY;
+}
+inline bool staged_pays(const Geometry &g, int K, bool f32) {
+    if (!f32) return g.T > 8 && g.T % 8 != 0 && (g.BN <= 65536 || g.BN >= 1000000);
+    return K == 8 || g.BN * K * g.T * (int64_t)sizeof(float) > 90000000;
+}
+
 template <int K, int G, int PSI, int XT, int LAYOUT>
 cudaError_t launch_forward(const FwdArgs &a, int blocks, cudaStream_t s, int *resident) {
     using T = typename XType<XT>::type;
@@ -2547,11 +2567,8 @@ cudaError_t launch_forward(const FwdArgs &a, int blocks, cudaStream_t s, int *re
                                    chunk_fwd_bytes<typename XI::Raw>(kChunkFwdThreads) +
                                        kappa_smem_bytes(a.p.mask_mode, KT / G, kChunkFwdThreads), s, resident);
     }
-    if constexpr (LAYOUT == 1 && K == 8 && XT == 0) {
-        // 8 float32 compartments, warps of 32 consecutive positions: staged per warp in 16-byte
-        // copies; the twin forward's 8-byte ones measured slower (T = 64, G = 2, 524288 neurons:
-        // 193 -> 210 us; T = 6, G = 1, 1048576 neurons: 37.5 -> 39.8 us)
-        if (a.g.inner % 32 == 0 && a.g.TXn % 32 == 0) {
+    if constexpr (LAYOUT == 1 && staged_forward<K, G, PSI, XT>()) {
+        if (a.g.inner % 32 == 0 && a.g.TXn % 32 == 0 && staged_pays(a.g, K, XT == 0)) {
             const size_t smem = (size_t)kFwdDepth * NT * K * sizeof(T) +
                                 kappa_smem_bytes(a.p.mask_mode, K / G, NT);
             return launch_or_query(dendsn_forward_staged_kernel<K, G, PSI, T>, a, blocks, NT, smem,

@@ -121,9 +121,11 @@ def test_element_aligned_outputs_get_the_same_bits(T, dtype, inner, spike_offset
     assert torch.equal(s, s0) and torch.equal(v, v0)
 
 
-# layers just beyond the sizes from which rows of a few steps take the twin backward: the same bits per neuron as the compartments-innermost layer
+# layers just beyond the sizes from which rows of a few steps take the twin backward, and from which
+# the forward is staged: the same bits per neuron as the compartments-innermost layer
 @pytest.mark.parametrize("T,B,K,G,dtype,psi", [
-    (2, 150, 8, 1, "bf16", "mh"), (3, 100, 8, 2, "bf16", "mh"), (1, 600, 8, 2, "bf16", "mh"), (1, 300, 8, 4, "f32", "mh")])
+    (2, 150, 8, 1, "bf16", "mh"), (3, 100, 8, 2, "bf16", "mh"), (1, 600, 8, 2, "bf16", "mh"), (1, 300, 8, 4, "f32", "mh"),
+    (6, 260, 4, 4, "f32", "mh"), (9, 16, 8, 2, "bf16", "identity"), (9, 260, 8, 2, "bf16", "identity")])
 def test_large_layers_bitwise(T, B, K, G, dtype, psi):
     w = workloads.Workload("twinl", T=T, B=B, N=4096, K=K, G=G, C=64, inner=64, dtype=dtype, psi=psi,
                            reset="hard", seed=T)

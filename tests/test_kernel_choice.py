@@ -37,3 +37,26 @@ def test_the_paper_layouts_backward(fake, T, N, inner, B, K, G, dtype, want):
     # never with dL/dS that is aligned for an element but not for a pair
     if want == TWIN:
         assert fake.launches(cfg, gs=(1 << 20) + (2 if dtype == "bf16" else 4))[1] != TWIN
+
+
+TWF, TWC, STAGED, PLAIN, CHUNK = ("dendsn_forward_twin_kernel", "dendsn_forward_twin_chunk_kernel",
+                                  "dendsn_forward_staged_kernel", "dendsn_forward_kernel", "dendsn_forward_chunk_kernel")
+
+
+@pytest.mark.parametrize("T,N,inner,B,K,G,dtype,psi,want", [
+    (6, 4096, 64, 10, 4, 2, "bf16", "mh", TWC), (6, 4096, 64, 10, 4, 2, "f32", "mh", TWF),
+    (6, 4000, 50, 10, 8, 2, "f32", "mh", TWF), (6, 4096, 64, 10, 8, 2, "f32", "mh", STAGED),
+    (6, 4096, 64, 200, 4, 4, "f32", "mh", TWF), (6, 4096, 64, 260, 4, 4, "f32", "mh", STAGED),
+    (6, 4000, 50, 260, 4, 4, "f32", "mh", TWF), (6, 4096, 64, 260, 4, 2, "f32", "mh", TWF),
+    (9, 4096, 64, 16, 8, 2, "bf16", "identity", STAGED), (16, 4096, 64, 16, 8, 2, "bf16", "identity", TWC),
+    (9, 4096, 64, 40, 8, 2, "bf16", "identity", TWC), (9, 4096, 64, 260, 8, 2, "bf16", "identity", STAGED),
+    (9, 4096, 64, 16, 8, 2, "bf16", "mh", TWC), (9, 4000, 50, 16, 8, 2, "bf16", "identity", TWC),
+])
+def test_the_paper_layouts_forward(fake, T, N, inner, B, K, G, dtype, psi, want):
+    cfg = binding.make_config(T, B, N, K, G, N // inner, inner, dtype, psi, layout="paper")
+    assert fake.launches(cfg)[0] == want
+    if want in (TWF, TWC):                       # spikes or V^s aligned for an element but not for a pair
+        A = 1 << 20
+        assert fake.launches(cfg, spikes=A + (2 if dtype == "bf16" else 4))[0] not in (TWF, TWC)
+        assert fake.launches(cfg, v_out=A + 4)[0] not in (TWF, TWC)
+        assert fake.launches(cfg, v_out=A)[0] == want
