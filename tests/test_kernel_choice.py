@@ -60,3 +60,11 @@ def test_the_paper_layouts_forward(fake, T, N, inner, B, K, G, dtype, psi, want)
         assert fake.launches(cfg, spikes=A + (2 if dtype == "bf16" else 4))[0] not in (TWF, TWC)
         assert fake.launches(cfg, v_out=A + 4)[0] not in (TWF, TWC)
         assert fake.launches(cfg, v_out=A)[0] == want
+
+
+@pytest.mark.parametrize("T,B,K,want", [
+    (12, 6, 16, CHUNK), (12, 7, 16, PLAIN), (12, 64, 8, CHUNK), (12, 65, 8, PLAIN), (8, 6, 16, PLAIN),
+    (12, 512, 4, CHUNK), (12, 513, 4, PLAIN), (12, 600, 2, CHUNK),
+])
+def test_the_forward_in_chunks(fake, T, B, K, want):
+    assert fake.launches(binding.make_config(T, B, 4096, K, 1, 64, 64))[0] == want
