@@ -160,13 +160,14 @@ def dendsn_workspace_size(cfg: dendsn_config):
     return int(s.value), int(w.value)
 
 
-# Bytes a config makes the kernels touch in each tensor, by the config's value and the current
-# device (scratch_bytes follows the device's residency). Bounded: forgotten when it has grown.
+# Bytes a config makes the kernels touch in each tensor, by the fields that decide them. Bounded:
+# forgotten when it has grown. The workspace's sizes are not among them: the library plans them
+# by what its kernels' residency queries answer, and an answer may differ from an earlier one.
 _needs = {}
 
 
 def _config_needs(cfg) -> dict:
-    key = (bytes(cfg), torch.cuda.current_device() if torch.cuda.is_initialized() else -1)
+    key = (cfg.T, cfg.B, cfg.N, cfg.K, cfg.G, cfg.C, cfg.x_dtype, cfg.mask_per_neuron)
     n = _needs.get(key)
     if n is None:
         T, B, N, K, C, Kb = cfg.T, cfg.B, cfg.N, cfg.K, cfg.C, cfg.K // cfg.G
@@ -178,19 +179,22 @@ def _config_needs(cfg) -> dict:
              "zeta": C * Kb * 4, "kappa": C * Kb * 4, "grad_zeta": C * Kb * 4,
              "grad_kappa": C * Kb * 4, "mask": (N if cfg.mask_per_neuron else C) * Kb,
              "grad_beta": C * 4}
-        n["saved"], n["scratch"] = dendsn_workspace_size(cfg)
         if len(_needs) >= 256:
             _needs.clear()
         _needs[key] = n
     return n
 
 
-def _need(cfg, **tensors):
+def _need(cfg, saved=None, scratch=None, **tensors):
     """Refuses on the host any tensor smaller than what the config makes the kernels touch."""
     needs = _config_needs(cfg)
     for name, t in tensors.items():
         if t is not None and t.nbytes < needs[name]:
             raise ValueError(f"{name}: {t.nbytes} bytes, the config needs {needs[name]}")
+    if saved is not None or scratch is not None:
+        for name, t, need in zip(("saved", "scratch"), (saved, scratch), dendsn_workspace_size(cfg)):
+            if t is not None and t.nbytes < need:
+                raise ValueError(f"{name}: {t.nbytes} bytes, the config needs {need}")
 
 
 def dendsn_forward(cfg, x, alpha, xi, zeta, kappa, mask, spikes, v_out=None, saved=None,

@@ -2,6 +2,7 @@
 import threading
 
 import pytest
+import torch
 
 from paper_2412_06355_gb300 import binding
 
@@ -60,3 +61,16 @@ def test_a_failed_opt_in_is_an_error_and_not_remembered(fake):
     with pytest.raises(AssertionError):
         fake.launches(cfg)
     assert fake.launches(cfg)[0] == "tp_forward_kernel"
+
+
+def test_the_bindings_check_follows_the_plan(fake, monkeypatch):
+    """The binding checks a workspace against the plan that the library has now, not against the one
+    that it made while a query failed."""
+    monkeypatch.setattr(binding, "_lib", fake.lib)
+    cfg = binding.make_config(4, 64, 131072, 4, 1, 128, 1024, layout="paper")
+    fake.lib.fake_fail_queries(2)
+    binding._need(cfg, scratch=torch.empty(1 << 26, dtype=torch.uint8))       # planned while they fail
+    now = in_another_thread(lambda: binding.dendsn_workspace_size(cfg))[1]
+    binding._need(cfg, scratch=torch.empty(now, dtype=torch.uint8))
+    with pytest.raises(ValueError, match="scratch"):
+        binding._need(cfg, scratch=torch.empty(now - 16, dtype=torch.uint8))
