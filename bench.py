@@ -154,7 +154,8 @@ class ClockSampler:
 
 # ------------------------------------------------------------------ kernel names
 def kernel_names(w):
-    """(forward, backward) kernels the library launches for workload w, following its plan:
+    """(forward, backward) one-neuron-per-thread kernels of workload w (or the time-parallel ones)
+    by the library's plan, before the chunk and twin kernels take their layers (launched_kernels):
     narrow long-horizon layers take the time-parallel kernels; rows of one full chunk
     (T = 4 or 8) whose 8 compartments sit on one lane, compartments innermost and no
     residual term, take the phased backward (one lane per neuron: bf16, or float32 with
@@ -175,6 +176,58 @@ def kernel_names(w):
     if w.K == 8 and w.G == 1 and w.dtype == "f32" and w.T == 4 and not w.residual:
         return fwd, "dendsn_backward_rowpair_kernel"
     return fwd, "dendsn_backward_kernel"
+
+
+def _twin_backward(w, f32, KT):
+    """Whether the paper layout's backward runs two neighbouring neurons per thread."""
+    n_ck = (w.T + 7) // 8 - 1 if w.T > 4 else 0
+    lanes = w.B * w.N * (w.K // KT)
+    if (w.psi != "mh" and w.G > 1) or (w.G == 4 and w.T > 4):
+        return False
+    if w.inner < 8 and (w.T <= 4 or (f32 and (w.K == 8 or (w.G > 1 and w.T > 8))) if KT == 8
+                        else KT == 4 and f32 and w.G == 1 and w.K != 8):
+        return False
+    if KT < 8:
+        return not (f32 and n_ck > 0)
+    if w.T == 1:
+        return w.G > (2 if f32 else 1) and lanes > (2100000 if w.G == 2 else 1000000)
+    if not f32 and w.T < 4:
+        return lanes * w.T > 1200000
+    if f32 and w.G == 1 and w.T == 9:
+        return False
+    whole = w.T == 4 if w.T <= 4 else w.T == 6 or w.T % 8 == 0 or w.T >= 32
+    return lanes > (24576 if whole else 131072)
+
+
+def launched_kernels(w):
+    """(forward, backward) kernels the library launches for workload w with aligned tensors and the
+    saved buffer, following its plan and dispatch rules: the time-parallel kernels for narrow
+    long-horizon layers whose series fit in shared memory; the forward in chunks for most rows of
+    more than 8 steps; for the paper layout with an even H*W the twin kernels (the forward staged
+    per warp in some float32 and identity layers); the one-neuron kernels for the rest."""
+    BN, f32 = w.B * w.N, w.dtype == "f32"
+    if w.T >= 256 and BN <= 2048 and 4 * w.T * (w.K + 5) <= 200 * 1024:
+        return "tp_forward_kernel", "tp_backward_kernel"
+    paper = w.layout == "paper" and w.K > 1 and w.inner > 1
+    fwd, bwd = "dendsn_forward_kernel", "dendsn_backward_kernel"
+    if w.T < 256 or BN > 2048:
+        bwd = kernel_names(w)[1]
+    chunk_line = {16: 24576, 8: 262144, 4: 2097152}.get(w.K, BN)
+    if w.T > 8 and ((w.inner % 2 == 1 and f32) if paper else (w.K > 1 or f32)) and \
+            not (f32 and BN > chunk_line):
+        fwd = "dendsn_forward_chunk_kernel"
+    elif paper and w.inner % 2 == 0:
+        if f32:
+            staged = w.K == 8 or (w.K == w.G == 4 and BN * w.K * w.T * 4 > 90000000)
+        else:
+            staged = w.K == 8 and w.G == 2 and w.psi != "mh" and w.T > 8 and w.T % 8 != 0 and \
+                (BN <= 65536 or BN >= 1000000)
+        fwd = "dendsn_forward_staged_kernel" if staged and w.inner % 32 == 0 else \
+            "dendsn_forward_twin_kernel" if f32 else "dendsn_forward_twin_chunk_kernel"
+    KT = 4 if f32 and w.K >= 8 and w.G == 1 and w.T <= 4 else min(w.K, 8)
+    if paper and w.inner % 2 == 0 and bwd != "dendsn_backward_rowpair_kernel" and _twin_backward(w, f32, KT):
+        bwd = "dendsn_backward_twin_short_kernel" if w.T <= 4 and KT < 8 else "dendsn_backward_twin_kernel"
+    return fwd, bwd
 
 
 # ------------------------------------------------------------------ traffic record
@@ -681,7 +734,7 @@ def layer_report(layer, timing, world, dev, peak, peak_kind, clock):
     ab = w.algorithmic_bytes()
     ops = w.fp32_ops_per_neuron_step()
     fwd_avg, bwd_avg = statistics.mean(timing["fwd_ms"]), statistics.mean(timing["bwd_ms"])
-    fname, bname = kernel_names(w)
+    fname, bname = launched_kernels(w)
     if bwd_avg >= fwd_avg:
         kname, kbytes, kms, kops = bname, ab["backward"], bwd_avg, ops["backward"]
     else:
