@@ -329,7 +329,7 @@ dendsn_status compute_plan(const dendsn_config &c, Plan *pl, bool *sized) {
     tile_columns(pl->gf, nt_f, c.K / KT);
     tile_columns(pl->gb, bwd_threads(KTB), c.K / KTB);
     // narrow layers with long horizons: one block per neuron, time scanned in parallel
-    pl->tp = c.T >= kTpMinT && BN <= kTpMaxNeurons && tp_smem_bytes(c.T, c.K, true) <= kTpMaxSmem;
+    pl->tp = c.T >= kTpMinT && BN <= kTpMaxNeurons && tp_smem_bytes(c.T, c.K) <= kTpMaxSmem;
     // blocks of the forward and backward kernels that fit on one SM. The backward's is taken
     // for the build without dL/dbeta, so that both builds of a layer share one tiling (and sum
     // the parameter gradients in the same order); the two layouts of a layer share it only

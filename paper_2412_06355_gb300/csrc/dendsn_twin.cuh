@@ -391,12 +391,13 @@ struct TwinSmem {
     }
 };
 // Resident blocks the register cap leaves room for: 64-thread blocks (8-compartment lanes) six
-// at 168 registers; 128-thread blocks four at 128 registers, or three where that spills (four
-// compartments per branch, or a build with both loops of an 8-step chunk) or where the shared
-// memory of 8 float32 steps allows no more.
-template <int KT, int G, typename XT, int LC, bool FULL>
+// at 168 registers; 128-thread blocks three in the builds with both loops of an 8-step chunk and where
+// the shared memory of 8 float32 steps allows no more, else four at 128 registers. Spills that are
+// left (bytes stored and loaded, Mexican hat, bfloat16, K = 4, G = 2): 72 and 128 with complete 8-step
+// chunks, 48 and 84 with both loops, 4 and 4 at T = 6.
+template <int KT, typename XT, int LC, bool FULL>
 constexpr int twin_min_blocks() {
-    return KT == 8 ? 6 : (G == 4 || (LC == 8 && (!FULL || sizeof(XT) == 4)) ? 3 : 4);
+    return KT == 8 ? 6 : (LC == 8 && (!FULL || sizeof(XT) == 4) ? 3 : 4);
 }
 
 // The backward in chunks of up to LC steps (L: the plan's chunk length; LC = L, or the number
@@ -413,7 +414,7 @@ constexpr int twin_min_blocks() {
 // one group each, and phase 1 of the next chunk waits for them one by one.
 template <int K, int G, int PSI, typename XT, int L, int LC, bool FULL>
 __global__ void __launch_bounds__(bwd_threads(bwd_lane_compartments(K, G, xt_code<XT>(), L)) / 2,
-                                  twin_min_blocks<bwd_lane_compartments(K, G, xt_code<XT>(), L), G, XT, LC, FULL>())
+                                  twin_min_blocks<bwd_lane_compartments(K, G, xt_code<XT>(), L), XT, LC, FULL>())
 dendsn_backward_twin_kernel(const BwdArgs A) {
     pdl_wait();
     constexpr int KT = bwd_lane_compartments(K, G, xt_code<XT>(), L);
@@ -692,6 +693,8 @@ dendsn_backward_twin_kernel(const BwdArgs A) {
                             vd[tt][q] = v;
                         });
                     }
+                    // into the slots just read: the copies are volatile and clobber memory, so they
+                    // stay behind the reads above without an operand that depends on them
                     if (more) fetch_x(in, cn, u);
                     cp_async_commit();
                     if (live) {

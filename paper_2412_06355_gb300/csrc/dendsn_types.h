@@ -159,7 +159,7 @@ cudaError_t launch_finalize(const FinArgs &a, cudaStream_t s);
 constexpr int kTpMinT = 256;
 constexpr int64_t kTpMaxNeurons = 2048;
 constexpr size_t kTpMaxSmem = 200 * 1024;
-size_t tp_smem_bytes(int T, int K, bool backward);
+size_t tp_smem_bytes(int T, int K);
 template <int K, int G, int XT>
 cudaError_t launch_forward_tp(const FwdArgs &a, int psi, int layout, cudaStream_t s);
 template <int K, int G, int XT>

@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(256, 2) lif_backward_kernel(const LifArgs A) {
 // in no more registers. Same operations, same bits. GB300, us: T = 8, 8.4M neurons 198 -> 163,
 // T = 64 bfloat16, 2.1M neurons 362 -> 206, T = 16 bfloat16, 786k neurons 36 -> 22; small layers
 // and ragged short rows, where the compiler's own order of the other kernel's loads does better,
-// stay there (T = 12, 80k neurons 5.8 -> 7.1; T = 5, 1M neurons 11 -> 14).
+// stay there (T = 12, 80k neurons 5.8 -> 7.1; T = 5, 1M neurons 11 -> 14). Either side of the line:
+// bfloat16 T = 16, 500000 neurons 22.0 on the other kernel, 524288 15.4; float32 26.4 and 23.8.
 constexpr int64_t kLifStreamM = 524288;
 template <typename XT, int VEC>
 __global__ void __launch_bounds__(256, 2) lif_backward_stream_kernel(const LifArgs A) {

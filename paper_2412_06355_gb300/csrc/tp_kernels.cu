@@ -715,10 +715,9 @@ cudaError_t tp_launch(void (*kernel)(Par...), unsigned blocks, unsigned threads,
 
 }  // namespace
 
-// The bytes by which the plan decides between these kernels and the chunked ones.
-size_t tp_smem_bytes(int T, int K, bool backward) {
-    return sizeof(float) * (size_t)T * ((size_t)K + (backward ? 5 : 1));
-}
+// The bytes by which the plan decides between these kernels and the chunked ones: the backward's
+// planes without their padding to whole segments, which adds 2.6 KB at most to the plan's 200.
+size_t tp_smem_bytes(int T, int K) { return sizeof(float) * (size_t)T * ((size_t)K + 5); }
 
 template <int K, int G, int XT>
 cudaError_t launch_forward_tp(const FwdArgs &a, int psi, int layout, cudaStream_t s) {
