@@ -243,6 +243,11 @@ const char *dendsn_last_error(void);
 /* Number of kernels the library enqueued since load (all threads). */
 uint64_t dendsn_launch_count(void);
 
+/* Number of plans made since load (all threads) while a residency query failed (no device, or a
+   transient error). The workspace sizes of such a plan need not be those of the next one: a caller
+   that remembers sizes remembers only those that were answered with this number unchanged. */
+uint64_t dendsn_unsized_plan_count(void);
+
 #ifdef __cplusplus
 }
 #endif

@@ -121,6 +121,8 @@ def load() -> ctypes.CDLL:
             lib.dendsn_last_error.restype = ctypes.c_char_p
             lib.dendsn_launch_count.argtypes = []
             lib.dendsn_launch_count.restype = ctypes.c_uint64
+            lib.dendsn_unsized_plan_count.argtypes = []
+            lib.dendsn_unsized_plan_count.restype = ctypes.c_uint64
             _lib = lib
     return _lib
 
@@ -160,14 +162,14 @@ def dendsn_workspace_size(cfg: dendsn_config):
     return int(s.value), int(w.value)
 
 
-# Bytes a config makes the kernels touch in each tensor, by the fields that decide them. Bounded:
-# forgotten when it has grown. The workspace's sizes are not among them: the library plans them
-# by what its kernels' residency queries answer, and an answer may differ from an earlier one.
+# Bytes a config makes the kernels touch in each tensor, by the config's value and the current
+# device (scratch_bytes follows the device's residency). Bounded: forgotten when it has grown. Not
+# kept while a residency query failed: the sizes of the next plan may be others.
 _needs = {}
 
 
 def _config_needs(cfg) -> dict:
-    key = (cfg.T, cfg.B, cfg.N, cfg.K, cfg.G, cfg.C, cfg.x_dtype, cfg.mask_per_neuron)
+    key = (bytes(cfg), torch.cuda.current_device() if torch.cuda.is_initialized() else -1)
     n = _needs.get(key)
     if n is None:
         T, B, N, K, C, Kb = cfg.T, cfg.B, cfg.N, cfg.K, cfg.C, cfg.K // cfg.G
@@ -179,22 +181,21 @@ def _config_needs(cfg) -> dict:
              "zeta": C * Kb * 4, "kappa": C * Kb * 4, "grad_zeta": C * Kb * 4,
              "grad_kappa": C * Kb * 4, "mask": (N if cfg.mask_per_neuron else C) * Kb,
              "grad_beta": C * 4}
-        if len(_needs) >= 256:
-            _needs.clear()
-        _needs[key] = n
+        unsized = load().dendsn_unsized_plan_count()
+        n["saved"], n["scratch"] = dendsn_workspace_size(cfg)
+        if load().dendsn_unsized_plan_count() == unsized:
+            if len(_needs) >= 256:
+                _needs.clear()
+            _needs[key] = n
     return n
 
 
-def _need(cfg, saved=None, scratch=None, **tensors):
+def _need(cfg, **tensors):
     """Refuses on the host any tensor smaller than what the config makes the kernels touch."""
     needs = _config_needs(cfg)
     for name, t in tensors.items():
         if t is not None and t.nbytes < needs[name]:
             raise ValueError(f"{name}: {t.nbytes} bytes, the config needs {needs[name]}")
-    if saved is not None or scratch is not None:
-        for name, t, need in zip(("saved", "scratch"), (saved, scratch), dendsn_workspace_size(cfg)):
-            if t is not None and t.nbytes < need:
-                raise ValueError(f"{name}: {t.nbytes} bytes, the config needs {need}")
 
 
 def dendsn_forward(cfg, x, alpha, xi, zeta, kappa, mask, spikes, v_out=None, saved=None,

@@ -156,6 +156,7 @@ namespace {
 
 thread_local char g_last_error[512] = "";
 std::atomic<uint64_t> g_launches{0};
+std::atomic<uint64_t> g_unsized{0};      // plans made while a residency query failed
 
 dendsn_status fail(dendsn_status st, const char *fmt, ...) {
     va_list ap;
@@ -427,8 +428,9 @@ dendsn_status make_plan(const dendsn_config *cfg, Plan *pl) {
             return DENDSN_OK;
         }
     }
-    bool sized = false;
+    bool sized = true;
     const dendsn_status st = compute_plan(*cfg, pl, &sized);
+    if (!sized) g_unsized.fetch_add(1);
     if (st == DENDSN_OK && sized && dev >= 0) {
         kept[at] = Kept{*cfg, dev, *pl};
         at = (at + 1) % kKept;
@@ -689,6 +691,8 @@ const char *dendsn_status_string(dendsn_status status) {
 const char *dendsn_last_error(void) { return g_last_error; }
 
 uint64_t dendsn_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
+
+uint64_t dendsn_unsized_plan_count(void) { return g_unsized.load(); }
 
 }  // extern "C"
 

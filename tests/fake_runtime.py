@@ -30,6 +30,7 @@ class Library:
         lib.dendsn_workspace_size.argtypes = [cfgp] + [ctypes.POINTER(ctypes.c_size_t)] * 2
         lib.dendsn_forward.argtypes = [cfgp] + [P] * 10
         lib.dendsn_backward.argtypes = [cfgp] + [P] * 16
+        lib.dendsn_unsized_plan_count.restype = ctypes.c_uint64
         lib.fake_launched.restype = ctypes.c_char_p
 
     def sizes(self, cfg):
