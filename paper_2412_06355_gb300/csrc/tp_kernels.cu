@@ -316,8 +316,10 @@ __device__ __forceinline__ float tp_charge(float z, float v, float beta, float t
 // horizon costs no more this way than a guess and its rounds. One thread runs it: it reads Z two vectors ahead of the
 // words it overwrites, so a second thread running the same loop could find V^s where it expects Z
 // (nothing orders the lanes of a warp). The barrier after it publishes V^s.
+// Not inlined: its copies (both resets, both callers) cost every layer instruction fetches (T = 2048,
+// one neuron, backward, against the kernel with one caller's copies: 1.01 times with both, 0.97 so).
 template <bool SOFT>
-__device__ __forceinline__ void tp_soma_serial(int T, float beta, float theta, float *vs) {
+__device__ __noinline__ void tp_soma_serial(int T, float beta, float theta, float *vs) {
     float v = SOFT && theta <= 0.f ? theta : 0.f;      // the state before a first step (tp_soma_run)
     float4 *p = reinterpret_cast<float4 *>(vs);        // planes hold a whole number of 32 steps
     float4 a = p[0], b = p[1];
